@@ -41,9 +41,9 @@ def listed():
         dict(name="vb_windows", kind="windows", n=1 << 20, c=4.0, R=2, T=1.0, sweeps=32),
         # the headline graph
         dict(name="vb_large", kind="vb", n=1 << 22, c=4.0, R=2, T=1.0, sweeps=64),
-        # uneven graphs in lock-step
-        dict(name="vb_batch", kind="vb_batch", count=48, lo=10.0, hi=18.0, c=4.0, R=2, T=1.0,
-             sweeps=32),
+        # uneven graphs in lock-step, the configurations read back
+        dict(name="vb_batch", kind="vb_batch", count=32, lo=10.0, hi=17.0, c=4.0, R=2, T=1.0,
+             sweeps=128, spins=True),
         # the headline SK sample: 256 replicas sharing the couplings
         dict(name="sk_large", kind="sk", n=8192, R=256, T=0.4, block=128, sweeps=64),
         # a small SK sample of odd size with few replicas
@@ -75,9 +75,12 @@ def draw(rng):
             d.update(c=rng.choice([3.0, 4.0, 4.0, 5.0]))
         return d
     if kind == "vb_batch":
+        d = dict(kind=kind, R=rng.choice([1, 2, 2, 4]), T=T, sweeps=_log_int(rng, 16, 128))
+        if rng.random() < 0.3:  # the graphs of one size of the bipartite ensemble, measured
+            lo = math.log2(_log_int(rng, 1 << 13, 1 << 16) // 2 * 2)
+            return dict(d, count=rng.randint(3, 16), lo=lo, hi=lo, z=4, spins=False)
         lo = rng.uniform(10.0, 12.0)
-        return dict(kind=kind, count=rng.randint(3, 64), lo=lo, hi=lo + rng.uniform(1.0, 6.0), c=4.0,
-                    R=rng.choice([1, 2, 2, 4]), T=T, sweeps=_log_int(rng, 8, 32))
+        return dict(d, count=rng.randint(3, 48), lo=lo, hi=lo + rng.uniform(1.0, 4.0), c=4.0, spins=True)
     if kind == "windows":
         return dict(kind=kind, n=_log_int(rng, 1 << 10, 1 << 20), c=4.0, R=rng.choice([2, 2, 4]), T=T,
                     sweeps=_log_int(rng, 16, 32))
@@ -137,7 +140,7 @@ def _regular(n, z, seed):
 
 def _graph(case, n, seed, k=0):
     gen = _generator(seed, k)
-    g = _regular(n, case["z"], seed) if "z" in case else _poisson(n, case["c"], gen)
+    g = _regular(n, case["z"], 64 * seed + k) if "z" in case else _poisson(n, case["c"], gen)
     g.update(seed=1000003 * seed + k, temps=[case["T"]] * case["R"])
     return g
 
@@ -205,6 +208,8 @@ def run(state):
     r.sweep(case["sweeps"])
     if kind == "windows":
         return r.windows()
+    if kind == "vb_batch" and case["spins"]:
+        return [s.view(np.int64) for s in r.spins()]
     if case.get("spins"):
         s = r.spins()
         return (*r.measure(), s if kind == "sk" else s[0].view(np.int64))
