@@ -169,8 +169,7 @@ struct VbPackedDev {
     const uint64_t* seeds;       // [n_graphs]
     const uint32_t* thr;         // [n_graphs][R][64]
     const uint4* groups;         // [n_groups] {first slice, slices, first entry, entries}
-    const uint4* slice_meta;     // [n_slices] {first entry, width, graph, upper}: upper =
-                                 // max entries to later colour classes | kind << 16
+    const uint4* slice_meta;     // [n_slices] {first entry, width, graph, 0}
     const uint32_t* group_graph; // [n_groups] graph of each group (groups never mix graphs)
     const uint8_t* gtab;         // [n_graphs] {uint32 thr[R][64]; uint64 seed; uint64 pad}
     const uint32_t* colour_groups;  // [n_colours+1] first group of each colour class
@@ -180,13 +179,16 @@ struct VbPackedDev {
     uint64_t* snap;              // [n_tw][n_slots][R]
     // upper entries for the energy: per slice, each lane's neighbours in later colour classes
     // (higher slots), sliced-ELL like col/jb; every edge appears once
-    const uint32_t* up_slice_base;  // [n_slices+1] (null: count over every directed entry)
+    const uint32_t* up_slice_base;  // [n_slices+1]
+    const uint32_t* up_row_slice;   // [up_rows] slice of each row of 32 upper entries
     const uint32_t* up_col;
     const uint64_t* up_jb;
+    uint32_t up_rows;
     int64_t n_slots;
     int32_t n_slices;
     int32_t R;
     int32_t n_colours;
+    int32_t n_graphs;
     uint64_t stage_wait_ns;      // bound of one pipeline wait in the colour kernel
 };
 
@@ -205,32 +207,27 @@ struct VbPlainDev {
     int32_t N, R, L;
 };
 
-// A measurement: per-lane counts of differences, accumulated with atomics into
-// dst[g * stride_g + r * stride_r + k * stride_k] (g graph, r replica or pair, k lane).
+// A measurement of the plain kernel: per-lane counts of differences, accumulated with atomics into
+// dst[r * stride_r + k * stride_k] (r replica or pair, k lane).
 //   kind 0: Hamming distance between the spins and snapshot w (all replicas)
 //   kind 1: Hamming distance between replicas 2p and 2p+1 (all pairs)
 //   kind 2: number of unsatisfied directed entries, J_ij s_i s_j = -1 (all replicas)
-// kind 0: C against snapshot w; 1: q; 2: E; 3 (packed only): C against snapshots 0 .. w-1 in
-// one pass (snapshot k adds at dst + k * stride_w), reading the current spins once
 struct VbCountJob {
     int kind;
     int w;
     int64_t* dst;
-    int64_t stride_g, stride_r, stride_k;
-    int64_t stride_w;
-    int shift;  // counts are added times 2^shift (the energy over upper entries counts each
-                // edge once and reports the number of unsatisfied directed entries, twice that)
+    int64_t stride_r, stride_k;
 };
 
-// slice_meta.w >> 16: how a slice's entries lie relative to its colour class (every entry of
-// every vertex goes to a later class / none does / some do)
-constexpr uint32_t kUpAll = 1u, kUpNone = 0u, kUpMixed = 2u;
-
-// The energy a measuring sweep takes of the state it starts from (one instance): per-lane
-// unsatisfied directed entries added at e_dst[r * stride_r + k * stride_k] (r replica, k lane).
-struct VbSweepMeas {
-    int64_t* e_dst;
-    int64_t stride_r, stride_k;
+// A measurement of the packed kernel, all its counts in one launch: C against snapshots 0 .. n_c - 1
+// (added at c + g c_g + r c_r + k c_k + w c_w: g graph, r replica, k lane), q (r a replica pair;
+// null: none) and the unsatisfied directed entries e (null: none).
+struct VbMeasure {
+    int n_c;
+    int64_t *c, *q, *e;
+    int64_t c_g, c_r, c_k, c_w;
+    int64_t q_g, q_r, q_k;
+    int64_t e_g, e_r, e_k;
 };
 
 // launch wrappers (vb_kernels.cu); each returns the number of kernel launches queued
@@ -245,19 +242,12 @@ int vb_packed_init(const VbPackedDev& d, cudaStream_t st);
 int vb_packed_sweep(const VbPackedDev& d, const uint32_t* colour_groups, const uint32_t* clock,
                     uint32_t t_off, int variant, bool fused, cudaStream_t st);
 constexpr int kVbColourVariants = 3;
-// The same sweep (same spins, same random numbers) that also adds the energy of the state it
-// starts from (vb_colour_meas.cu); single-instance layouts only.
-int vb_packed_sweep_meas(const VbPackedDev& d, const uint32_t* colour_groups,
-                         const uint32_t* clock, uint32_t t_off, int variant, bool fused,
-                         const VbSweepMeas& meas, cudaStream_t st);
 int vb_packed_snapshot(const VbPackedDev& d, int w, cudaStream_t st);
 // the upper entries (each vertex's neighbours in later colour classes, padded with the vertex
-// itself and J = 0) from col and jb, given up_slice_base
+// itself and J = 0) and their rows' slices, from col and jb, given up_slice_base
 int vb_packed_build_upper(const VbPackedDev& d, cudaStream_t st);
-// also_q (kind 1, with job of kind 0 or 3): the replica overlaps in the same launch, one more
-// pass over the warp's slices (whose current spins are still in L1)
-int vb_packed_count(const VbPackedDev& d, const VbCountJob& job, cudaStream_t st,
-                    const VbCountJob* also_q = nullptr);
+// one launch (vb_measure.cu); returns the launches queued, or -1
+int vb_packed_measure(const VbPackedDev& d, const VbMeasure& m, cudaStream_t st);
 
 int vb_plain_init(const VbPlainDev& d, cudaStream_t st);
 int vb_plain_colour(const VbPlainDev& d, int32_t v_begin, int32_t v_end, const uint32_t* clock,

@@ -220,10 +220,6 @@ public:
             }
         if (kernel == SG_VB_PACKED) build_packed();
         else build_plain();
-        // the energy of a measured state taken by the next sweep (one instance, packed);
-        // SG_VB_FUSED_MEAS=0 keeps the standalone energy kernel (the results are the same)
-        const char* fm = getenv("SG_VB_FUSED_MEAS");
-        fuse_e_ = kernel == SG_VB_PACKED && n_graphs == 1 && !(fm && fm[0] == '0' && !fm[1]);
         Carver c;
         carve(c);
         ws_bytes_ = c.off;
@@ -274,17 +270,6 @@ public:
             } else {
                 tune_variant(st, pinned ? *pin - '0' : -1, pinned_f ? *pin_f - '0' : -1);
                 if (!pinned && !pinned_f) remember_tuning();
-            }
-            if (fuse_e_) {
-                // one measuring sweep (into the scratch energy counts of sg_measure, cleared
-                // before each use) sets its kernel up before the first measurement; the initial
-                // spins are drawn again afterwards
-                check_cuda(cudaMemsetAsync(clock_dev, 0, 4, st), "memset");
-                const VbSweepMeas m{mE_, (int64_t)Lc_, 1};
-                const int n = vb_packed_sweep_meas(pk_, colour_group_.data(), clock_dev, 0, variant_,
-                                                   fused_, m, st);
-                if (n < 0) fail(SG_ECUDA, "measuring colour kernel launch failed");
-                launches += n + vb_packed_init(pk_, st);
             }
         } else {
             up((void*)pl_.row_ptr, h_row_ptr_.data(), h_row_ptr_.size() * 4);
@@ -402,24 +387,6 @@ public:
         }
     }
 
-    bool has_pending() const override { return pend_; }
-
-    void sweep_pending(uint32_t t_off, cudaStream_t st) override {
-        if (!pend_) return sweep(t_off, st);
-        pend_ = false;
-        const VbSweepMeas m{pend_job_.dst, pend_job_.stride_r, pend_job_.stride_k};
-        const int n = vb_packed_sweep_meas(pk_, colour_group_.data(), clock_dev, t_off, variant_,
-                                           fused_, m, st);
-        if (n < 0) fail(SG_ECUDA, "measuring colour kernel launch failed");
-        launches += n;
-    }
-
-    void flush_pending(cudaStream_t st) override {
-        if (!pend_) return;
-        pend_ = false;
-        run_job(pend_job_, st);
-    }
-
     void snapshot(int w, cudaStream_t st) override {
         if (kernel_ == SG_VB_PACKED) launches += vb_packed_snapshot(pk_, w, st);
         else if (vb_plain_snapshot(pl_, w, st) < 0) fail(SG_ECUDA, "snapshot copy failed");
@@ -429,30 +396,33 @@ public:
     void measure_into(int64_t* Cb, int64_t* Qb, int64_t* Eb, int64_t ncol, int64_t u, int64_t tau,
                       cudaStream_t st) {
         const int64_t ntw = (int64_t)tw.size();
-        int64_t active = 0;
-        while (active < ntw && tw[active] <= tau) ++active;
-        const VbCountJob qj{1, 0, Qb + u, (int64_t)(R / 2) * Lc_ * ncol, (int64_t)Lc_ * ncol, ncol, 0, 0};
-        if (kernel_ == SG_VB_PACKED && active > 0) {
-            // every active snapshot and the replica overlaps in one pass over the current spins
-            VbCountJob j{3, (int)active, Cb + u, (int64_t)R * Lc_ * ntw * ncol,
-                         (int64_t)Lc_ * ntw * ncol, ntw * ncol, ncol, 0};
-            launches += vb_packed_count(pk_, j, st, R >= 2 ? &qj : nullptr);
-        } else {
-            for (int64_t w = 0; w < active; ++w) {
-                VbCountJob j{0, (int)w, Cb + w * ncol + u, (int64_t)R * Lc_ * ntw * ncol,
-                             (int64_t)Lc_ * ntw * ncol, ntw * ncol, 0, 0};
-                run_job(j, st);
-            }
-            if (R >= 2) run_job(qj, st);
+        int active = 0;
+        while (active < (int)ntw && tw[active] <= tau) ++active;
+        VbMeasure m{};
+        m.n_c = active;
+        m.c = Cb + u;
+        m.c_w = ncol;
+        m.c_k = ntw * ncol;
+        m.c_r = (int64_t)Lc_ * m.c_k;
+        m.c_g = R * m.c_r;
+        m.q = R >= 2 ? Qb + u : nullptr;
+        m.q_k = ncol;
+        m.q_r = (int64_t)Lc_ * ncol;
+        m.q_g = (R / 2) * m.q_r;
+        m.e = Eb + u;
+        m.e_k = ncol;
+        m.e_r = (int64_t)Lc_ * ncol;
+        m.e_g = R * m.e_r;
+        if (kernel_ == SG_VB_PACKED) {
+            const int n = vb_packed_measure(pk_, m, st);
+            if (n < 0) fail(SG_ECUDA, "measurement launch failed");
+            launches += n;
+            return;
         }
-        const VbCountJob ej{2, 0, Eb + u, (int64_t)R * Lc_ * ncol, (int64_t)Lc_ * ncol, ncol, 0, 0};
-        if (fuse_e_) {
-            flush_pending(st);  // two measurements of one state (a schedule and a window)
-            pend_ = true;
-            pend_job_ = ej;
-        } else {
-            run_job(ej, st);
-        }
+        for (int w = 0; w < active; ++w)
+            launches += vb_plain_count(pl_, VbCountJob{0, w, m.c + w * m.c_w, m.c_r, m.c_k}, st);
+        if (m.q) launches += vb_plain_count(pl_, VbCountJob{1, 0, m.q, m.q_r, m.q_k}, st);
+        launches += vb_plain_count(pl_, VbCountJob{2, 0, m.e, m.e_r, m.e_k}, st);
     }
 
     void measure_scheduled(int u, int64_t tau, cudaStream_t st) override {
@@ -501,22 +471,10 @@ public:
     }
 
     void measure_now(int64_t tau, cudaStream_t st) override {
-        flush_pending(st);
-        const int64_t ntw = (int64_t)tw.size();
         check_cuda(cudaMemsetAsync(mC_, 0, nmC() * 8, st), "memset");
         check_cuda(cudaMemsetAsync(mQ_, 0, nmQ() * 8, st), "memset");
         check_cuda(cudaMemsetAsync(mE_, 0, nmE() * 8, st), "memset");
-        for (int64_t w = 0; w < ntw; ++w) {
-            if (tw[w] > tau) break;
-            VbCountJob j{0, (int)w, mC_ + w, (int64_t)R * Lc_ * ntw, (int64_t)Lc_ * ntw, ntw, 0};
-            run_job(j, st);
-        }
-        if (R >= 2) {
-            VbCountJob j{1, 0, mQ_, (int64_t)(R / 2) * Lc_, (int64_t)Lc_, 1, 0};
-            run_job(j, st);
-        }
-        VbCountJob j{2, 0, mE_, (int64_t)R * Lc_, (int64_t)Lc_, 1, 0};
-        run_job(j, st);
+        measure_into(mC_, mQ_, mE_, 1, 0, tau, st);
     }
 
     void read_scheduled(int64_t tau, int64_t* C, int64_t* q, int64_t* E, cudaStream_t st) override {
@@ -664,11 +622,6 @@ private:
         if (bytes) check_cuda(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, st), "D2H copy");
     }
 
-    void run_job(const VbCountJob& j, cudaStream_t st) {
-        if (kernel_ == SG_VB_PACKED) launches += vb_packed_count(pk_, j, st);
-        else launches += vb_plain_count(pl_, j, st);
-    }
-
     void carve(Carver& c) {
         clock_dev = c.take<uint32_t>(1);
         d_thr_ = c.take<uint32_t>(thr_.size());
@@ -687,6 +640,8 @@ private:
             pk_.jb = c.take<uint64_t>(h_jb_.size());
             pk_.seeds = c.take<uint64_t>(n_inst);
             pk_.up_slice_base = c.take<uint32_t>(h_up_base_.size());
+            pk_.up_row_slice = c.take<uint32_t>(up_entries_ / 32);
+            pk_.up_rows = (uint32_t)(up_entries_ / 32);
             pk_.up_col = c.take<uint32_t>(up_entries_);
             pk_.up_jb = c.take<uint64_t>(up_entries_);
             pk_.S = c.take<uint64_t>((size_t)n_slots_ * R);
@@ -695,6 +650,7 @@ private:
             pk_.n_slots = n_slots_;
             pk_.n_slices = (int32_t)(n_slots_ / 32);
             pk_.R = R;
+            pk_.n_graphs = n_inst;
             pk_.n_colours = (int32_t)colour_group_.size() - 1;
             // SG_TEST_STAGE_WAIT_NS shortens the colour kernel's pipeline waits: a test of the
             // timeout path (the kernel gives up, flags SG_ETIMEOUT and exits cleanly)
@@ -857,13 +813,11 @@ private:
         // upper entries (energy measurement): neighbours in later colour classes only
         h_up_base_.assign(n_slices + 1, 0);
         std::vector<int32_t> up_width(n_slices, 0);
-        std::vector<uint32_t> up_kind(n_slices, kUpNone);
         parallel_ranges(n_slices, [&](int64_t s0, int64_t s1) {
             for (int64_t s = s0; s < s1; ++s) {
                 const int b = (int)h_slice_graph_[s];
                 const Graph& g = graphs_[b];
                 int w = 0;
-                bool all = true;
                 for (int l = 0; l < 32; ++l) {
                     const int64_t slot = s * 32 + l;
                     const int32_t i = slot_graph_vertex[slot];
@@ -872,10 +826,8 @@ private:
                     for (int32_t k = g.row_ptr[i]; k < g.row_ptr[i + 1]; ++k)
                         n_up += slot_of_[b][g.col[k]] > slot;
                     w = std::max(w, n_up);
-                    all = all && n_up == g.row_ptr[i + 1] - g.row_ptr[i];
                 }
                 up_width[s] = w;
-                up_kind[s] = w == 0 ? kUpNone : all ? kUpAll : kUpMixed;
             }
         });
         int64_t up_entries = 0;
@@ -891,7 +843,7 @@ private:
             m.x = h_slice_base_[s];
             m.y = (h_slice_base_[s + 1] - h_slice_base_[s]) / 32;
             m.z = h_slice_graph_[s];
-            m.w = (uint32_t)up_width[s] | up_kind[s] << 16;
+            m.w = 0;
             h_slice_meta_[s] = m;
         }
         // staging groups: consecutive slices of one colour, <= 8 slices and <= 1024 entries;
@@ -932,9 +884,6 @@ private:
     }
 
     int kernel_ = SG_VB_PACKED;
-    bool fuse_e_ = false;  // the energy of a measured state is taken by the next sweep
-    bool pend_ = false;    // such a measurement is waiting for that sweep (pend_job_ its target)
-    VbCountJob pend_job_{};
     int variant_ = 0;     // colour-kernel pipeline shape chosen by the autotuner at attach
     bool fused_ = false;  // one cooperative launch per sweep (else one launch per colour class)
     int Lc_ = 64;

@@ -48,11 +48,6 @@ int vb_packed_init(const VbPackedDev& d, cudaStream_t st) {
     return 1;
 }
 
-int vb_packed_sweep(const VbPackedDev& d, const uint32_t* colour_groups, const uint32_t* clock,
-                    uint32_t t_off, int variant, bool fused, cudaStream_t st) {
-    return packed_sweep<false>(d, colour_groups, clock, t_off, variant, fused, VbSweepMeas{}, st);
-}
-
 // ---------------------------------------------------------------------------------------------
 // upper entries: one thread per slot keeps, in order, the entries whose neighbour lies in a
 // later colour class (a higher slot), and pads the rest of its upper width with itself
@@ -80,6 +75,8 @@ __global__ void k_vb_build_upper(VbPackedDev d) {
         up_col[ub + 32 * e2 + l] = (uint32_t)slot;
         up_jb[ub + 32 * e2 + l] = 0ull;
     }
+    uint32_t* row_slice = const_cast<uint32_t*>(d.up_row_slice);
+    for (uint32_t e = l; e < uw; e += 32) row_slice[(ub >> 5) + e] = (uint32_t)s;
 }
 
 int vb_packed_build_upper(const VbPackedDev& d, cudaStream_t st) {
@@ -111,246 +108,6 @@ static int copy_bytes(const void* src, void* dst, int64_t bytes, cudaStream_t st
 int vb_packed_snapshot(const VbPackedDev& d, int w, cudaStream_t st) {
     const int64_t words = d.n_slots * d.R;
     return copy_bytes(d.S, d.snap + (int64_t)w * words, words * 8, st);
-}
-
-// ---------------------------------------------------------------------------------------------
-// packed: per-lane difference counts (C, q, E).  Each warp walks a contiguous run of slices,
-// accumulates bit-sliced per-lane counters (16 planes) and flushes them to global memory when
-// the graph changes and at the end of its run.
-// ---------------------------------------------------------------------------------------------
-// A lane adds at most one word per slot (C, q: 16 slices, so 5 planes hold up to 31) or one per
-// entry (E: 16 slices x width <= 63 = 1008 words: 10 planes, up to 1023), so PL planes cannot
-// overflow before the flush at the end of a run; the 32-lane butterfly needs PL + 5 planes.
-constexpr int kCountSlicesPerWarp = 16;
-
-template <int NQ, int PW>
-__device__ __forceinline__ void count_add(uint64_t (&p)[NQ][PW], int q, uint64_t x) {
-#pragma unroll
-    for (int b = 0; b < PW - 5; ++b) {
-        const uint64_t c = p[q][b] & x;
-        p[q][b] ^= x;
-        x = c;
-    }
-}
-
-// Sum the bit-sliced counters of the 32 lanes with a butterfly of bit-sliced additions, then
-// lane l adds the totals of spin lanes l and l + 32.  With a CTA-shared accumulator (cta_acc,
-// [NQ][64], one graph per CTA run) the warp adds there and the CTA flushes once; otherwise
-// straight into global memory.
-template <int NQ, int PW>
-__device__ __forceinline__ void count_flush(uint64_t (&p)[NQ][PW], const VbCountJob& job,
-                                            uint32_t g, int nq, uint32_t lane,
-                                            unsigned long long* cta_acc = nullptr) {
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        if (q >= nq) break;
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            uint64_t carry = 0ull;
-#pragma unroll
-            for (int b = 0; b < PW; ++b) {
-                const uint64_t o = __shfl_xor_sync(0xFFFFFFFFu, p[q][b], off);
-                const uint64_t x = p[q][b] ^ o;
-                const uint64_t sum = x ^ carry;
-                carry = (p[q][b] & o) | (carry & x);
-                p[q][b] = sum;
-            }
-        }
-        uint32_t c0 = 0, c1 = 0;
-#pragma unroll
-        for (int b = 0; b < PW; ++b) {
-            c0 |= (uint32_t)((p[q][b] >> lane) & 1ull) << b;
-            c1 |= (uint32_t)((p[q][b] >> (lane + 32)) & 1ull) << b;
-        }
-        if (cta_acc) {
-            if (c0) atomicAdd(cta_acc + q * 64 + lane, (unsigned long long)c0);
-            if (c1) atomicAdd(cta_acc + q * 64 + lane + 32, (unsigned long long)c1);
-        } else {
-            int64_t* base = job.dst + g * job.stride_g + q * job.stride_r;
-            if (c0)
-                atomicAdd((unsigned long long*)(base + lane * job.stride_k),
-                          (unsigned long long)c0 << job.shift);
-            if (c1)
-                atomicAdd((unsigned long long*)(base + (lane + 32) * job.stride_k),
-                          (unsigned long long)c1 << job.shift);
-        }
-#pragma unroll
-        for (int b = 0; b < PW; ++b) p[q][b] = 0ull;
-    }
-}
-
-// EN: the energy job (kind 2, PW = 15); otherwise C and q jobs (kinds 0, 1, 3, PW = 10)
-template <int R, bool EN>
-__global__ void __launch_bounds__(256, EN ? (R <= 2 ? 2 : 1) : (R <= 2 ? 3 : 2))
-    k_vb_packed_count(VbPackedDev d, VbCountJob job, VbCountJob qjob) {
-    constexpr int NQ = R;
-    constexpr int PW = EN ? 15 : 10;
-    const uint32_t lane = threadIdx.x & 31u;
-    const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t s_lo = (int64_t)warp * kCountSlicesPerWarp;
-    int64_t s_hi = s_lo + kCountSlicesPerWarp;
-    if (s_hi > d.n_slices) s_hi = d.n_slices;
-    const int64_t words = d.n_slots * R;
-    // kind 3: one pass per snapshot over this warp's slices; the current spins of the slices
-    // (a few KB) stay in L1 after the first pass
-    const int main_passes = job.kind == 3 ? job.w : 1;
-    const int passes = main_passes + (!EN && qjob.kind == 1 ? 1 : 0);
-    // The CTA's slices belong to one graph (the common case: a single instance, or slices of
-    // one graph in a batch): the warps add into a shared accumulator and the CTA flushes it once,
-    // so the global counters see one atomic per CTA instead of one per warp.
-    __shared__ unsigned long long acc[NQ * 64];
-    __shared__ int one_graph;
-    const int64_t cta_lo = (int64_t)blockIdx.x * (blockDim.x / 32) * kCountSlicesPerWarp;
-    int64_t cta_hi = cta_lo + (int64_t)(blockDim.x / 32) * kCountSlicesPerWarp;
-    if (cta_hi > d.n_slices) cta_hi = d.n_slices;
-    if (threadIdx.x == 0)
-        one_graph = cta_lo < cta_hi && __ldg(d.slice_graph + cta_lo) == __ldg(d.slice_graph + cta_hi - 1);
-    for (int pass = 0; pass < passes; ++pass) {
-        VbCountJob jb = job;
-        if (pass >= main_passes) {
-            jb = qjob;
-        } else if (job.kind == 3) {
-            jb.kind = 0;
-            jb.w = pass;
-            jb.dst = job.dst + pass * job.stride_w;
-        }
-        const int kind = jb.kind;
-        const int nq = kind == 1 ? R / 2 : R;
-        uint64_t p[NQ][PW];
-#pragma unroll
-        for (int q = 0; q < NQ; ++q)
-#pragma unroll
-            for (int b = 0; b < PW; ++b) p[q][b] = 0ull;
-        const uint64_t* snap = d.snap + (int64_t)(kind == 0 ? jb.w : 0) * words;
-        int64_t cur_g = -1;
-        for (int q = threadIdx.x; q < NQ * 64; q += blockDim.x) acc[q] = 0ull;
-        __syncthreads();
-        unsigned long long* cta_acc = one_graph ? acc : nullptr;
-        if (cta_acc && s_lo < s_hi) {
-            // every slice of the CTA belongs to one graph: no per-slice graph test, so nothing
-            // but the loads and the counting sits in the loop and the loads of several slices
-            // (or entries) can be in flight together
-            cur_g = __ldg(d.slice_graph + s_lo);
-            if constexpr (!EN) {
-#pragma unroll 4
-                for (int64_t s = s_lo; s < s_hi; ++s) {
-                    const int64_t slot = s * 32 + lane;
-                    const SpinWords<R> si = load_words<R>(d.S + slot * R);
-                    if (kind == 0) {
-                        const SpinWords<R> sw = load_words<R>(snap + slot * R);
-#pragma unroll
-                        for (int r = 0; r < R; ++r) count_add<NQ, PW>(p, r, si.v[r] ^ sw.v[r]);
-                    } else {
-#pragma unroll
-                        for (int q = 0; q < R / 2; ++q)
-                            count_add<NQ, PW>(p, q, si.v[2 * q] ^ si.v[2 * q + 1]);
-                    }
-                }
-            } else {
-                uint32_t base = __ldg(d.slice_base + s_lo);
-                for (int64_t s = s_lo; s < s_hi; ++s) {
-                    const uint32_t next = __ldg(d.slice_base + s + 1);
-                    const SpinWords<R> si = load_words<R>(d.S + (s * 32 + lane) * R);
-                    const uint32_t width = (next - base) >> 5;
-                    uint32_t idx = base + lane;
-#pragma unroll 4
-                    for (uint32_t e = 0; e < width; ++e, idx += 32) {
-                        const uint32_t j = __ldg(d.col + idx);
-                        const uint64_t J = __ldg(d.jb + idx);
-                        const SpinWords<R> sj = gather_words<R>(d.S + (int64_t)j * R);
-#pragma unroll
-                        for (int r = 0; r < R; ++r) count_add<NQ, PW>(p, r, si.v[r] ^ sj.v[r] ^ J);
-                    }
-                    base = next;
-                }
-            }
-        } else
-        // padding slots hold zero words and zero couplings, so they add nothing: no vinfo test,
-        // and the loads of several slices can be in flight together
-#pragma unroll 4
-        for (int64_t s = s_lo; s < s_hi; ++s) {
-            const uint32_t g = __ldg(d.slice_graph + s);  // warp-uniform
-            if ((int64_t)g != cur_g) {
-                if (cur_g >= 0) count_flush<NQ, PW>(p, jb, (uint32_t)cur_g, nq, lane, cta_acc);
-                cur_g = g;
-            }
-            const int64_t slot = s * 32 + lane;
-            const SpinWords<R> si = load_words<R>(d.S + slot * R);
-            if constexpr (!EN) {
-                if (kind == 0) {
-                    const SpinWords<R> sw = load_words<R>(snap + slot * R);
-#pragma unroll
-                    for (int r = 0; r < R; ++r) count_add<NQ, PW>(p, r, si.v[r] ^ sw.v[r]);
-                } else {
-#pragma unroll
-                    for (int q = 0; q < R / 2; ++q)
-                        count_add<NQ, PW>(p, q, si.v[2 * q] ^ si.v[2 * q + 1]);
-                }
-            } else {
-                const uint32_t base = __ldg(d.slice_base + s);
-                const uint32_t width = (__ldg(d.slice_base + s + 1) - base) >> 5;
-                uint32_t idx = base + lane;
-#pragma unroll 4
-                for (uint32_t e = 0; e < width; ++e, idx += 32) {
-                    const uint32_t j = __ldg(d.col + idx);
-                    const uint64_t J = __ldg(d.jb + idx);
-                    const SpinWords<R> sj = gather_words<R>(d.S + (int64_t)j * R);
-#pragma unroll
-                    for (int r = 0; r < R; ++r) count_add<NQ, PW>(p, r, si.v[r] ^ sj.v[r] ^ J);
-                }
-            }
-        }
-        if (cur_g >= 0) count_flush<NQ, PW>(p, jb, (uint32_t)cur_g, nq, lane, cta_acc);
-        if (cta_acc) {
-            __syncthreads();
-            const int64_t g = (int64_t)__ldg(d.slice_graph + cta_lo);
-            for (int q = threadIdx.x; q < nq * 64; q += blockDim.x) {
-                const unsigned long long v = acc[q];
-                if (v)
-                    atomicAdd((unsigned long long*)(jb.dst + g * jb.stride_g + (q >> 6) * jb.stride_r +
-                                                    (q & 63) * jb.stride_k),
-                              v << jb.shift);
-            }
-            __syncthreads();
-        }
-    }
-}
-
-// The energy job (kind 2) runs over the upper entries when the layout has them: each edge once,
-// from its lower-colour endpoint (the higher slot), counted twice (shift 1).
-int vb_packed_count(const VbPackedDev& d, const VbCountJob& job_in, cudaStream_t st,
-                    const VbCountJob* also_q) {
-    VbCountJob job = job_in;
-    VbCountJob qjob{};
-    qjob.kind = -1;
-    if (also_q && job.kind != 2 && job.kind != 1 && also_q->kind == 1) qjob = *also_q;
-    VbPackedDev dd = d;
-    if (job.kind == 2 && d.up_slice_base) {
-        dd.slice_base = d.up_slice_base;
-        dd.col = d.up_col;
-        dd.jb = d.up_jb;
-        job.shift = 1;
-    }
-    const int bs = 256;
-    const int64_t warps = (d.n_slices + kCountSlicesPerWarp - 1) / kCountSlicesPerWarp;
-    const unsigned nb = (unsigned)((warps + (bs / 32) - 1) / (bs / 32));
-    const bool en = job.kind == 2;
-    switch (d.R) {
-        case 1:
-            if (en) k_vb_packed_count<1, true><<<nb, bs, 0, st>>>(dd, job, qjob);
-            else k_vb_packed_count<1, false><<<nb, bs, 0, st>>>(dd, job, qjob);
-            break;
-        case 2:
-            if (en) k_vb_packed_count<2, true><<<nb, bs, 0, st>>>(dd, job, qjob);
-            else k_vb_packed_count<2, false><<<nb, bs, 0, st>>>(dd, job, qjob);
-            break;
-        case 4:
-            if (en) k_vb_packed_count<4, true><<<nb, bs, 0, st>>>(dd, job, qjob);
-            else k_vb_packed_count<4, false><<<nb, bs, 0, st>>>(dd, job, qjob);
-            break;
-        default: return -1;
-    }
-    return 1;
 }
 
 // ---------------------------------------------------------------------------------------------
