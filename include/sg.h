@@ -274,14 +274,13 @@ int sg_sk_blocked_schedule(int32_t n, int32_t block, int32_t *ops, int32_t cap, 
  *   s  device int8[n_replicas*n], spins +-1, replica-major
  *   h  device int32[n_replicas*n], output, replica-major
  *   n  2..2048;  n_replicas a multiple of 16 in 16..128;  cuda_stream a cudaStream_t (or NULL)
- * The tensor-core operand images live in one static device array of about 5.3 MiB inside the
- * library (held by every GPU that loads it until the process exits); larger sizes return
- * SG_EINVAL.  J, s and h must be device memory of the current device.  The first call on a
- * device looks up that array's device address.  Every call reuses the array and clears what must
- * start at zero, so calls that overlap on the GPU (different streams or host threads) race with
- * each other: serialise them.  The call is queued on cuda_stream, synchronises that stream and
- * returns after its work completed; errors are reported like every other call (status code,
- * sg_last_error). */
+ * Larger sizes return SG_EINVAL.  J, s and h must be device memory of the current device; no
+ * alignment beyond that of their types is needed.  The operands pass through shared and tensor
+ * memory only; where h overlaps J or s the fields pass through one static device array of 1 MiB
+ * (held by every GPU that loads the library until the process exits), and such calls that overlap
+ * on the GPU (different streams or host threads) race with each other: serialise them.  The call
+ * is queued on cuda_stream, synchronises that stream and returns after its work completed; errors
+ * are reported like every other call (status code, sg_last_error). */
 int sg_sk_fields_noalloc(const int8_t *J, const int8_t *s, int32_t n, int32_t n_replicas,
                          int32_t *h, void *cuda_stream);
 

@@ -318,7 +318,7 @@ def sg_sk_blocked_schedule(n, block):
 def sg_sk_fields_noalloc(J_dev: int, s_dev: int, n: int, n_replicas: int, h_dev: int,
                          stream_handle: int):
     """Local fields h = J s for callers that cannot allocate device memory (device pointers in
-    and out; the library's fixed static scratch holds the tensor-core operand images)."""
+    and out)."""
     _check(_load().sg_sk_fields_noalloc(ctypes.c_void_p(J_dev), ctypes.c_void_p(s_dev), int(n),
                                         int(n_replicas), ctypes.c_void_p(h_dev),
                                         ctypes.c_void_p(stream_handle)))
