@@ -242,6 +242,9 @@ int vb_packed_init(const VbPackedDev& d, cudaStream_t st);
 int vb_packed_sweep(const VbPackedDev& d, const uint32_t* colour_groups, const uint32_t* clock,
                     uint32_t t_off, int variant, bool fused, cudaStream_t st);
 constexpr int kVbColourVariants = 3;
+// words [lo, hi) of the configuration in the caller's order (graph_words: first word of each graph)
+int vb_packed_spins(const VbPackedDev& d, const int64_t* graph_words, int64_t lo, int64_t hi,
+                    uint64_t* out, cudaStream_t st);
 int vb_packed_snapshot(const VbPackedDev& d, int w, cudaStream_t st);
 // the upper entries (each vertex's neighbours in later colour classes, padded with the vertex
 // itself and J = 0) and their rows' slices, from col and jb, given up_slice_base

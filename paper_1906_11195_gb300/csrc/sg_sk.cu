@@ -407,14 +407,10 @@ public:
     size_t spins_bytes() const override { return (size_t)R * n_; }
 
     void get_spins(void* dst, cudaStream_t st) override {
-        const int words = Np_ / 32;
-        std::vector<uint32_t> S((size_t)R * words);
-        down(S.data(), d_.S, S.size() * 4, st);
+        launches += sk_spins(d_, d_spins_, st);
+        check_cuda(cudaGetLastError(), "spins launch");
+        down(dst, d_spins_, spins_bytes(), st);
         check_cuda(cudaStreamSynchronize(st), "read spins");
-        int8_t* out = static_cast<int8_t*>(dst);
-        for (int r = 0; r < R; ++r)
-            for (int i = 0; i < n_; ++i)
-                out[(size_t)r * n_ + i] = ((S[(size_t)r * words + i / 32] >> (i & 31)) & 1u) ? -1 : 1;
     }
 
     std::vector<uint32_t> thresholds() const override {
@@ -597,6 +593,7 @@ private:
         d_.flips = c.take<uint32_t>(kernel_ == SG_SK_BLOCKED ? (size_t)R * words : 0);
         d_.snap = c.take<uint32_t>((size_t)R * words * tw.size());
         d_.err = c.take<int>(1);
+        d_spins_ = c.take<int8_t>((size_t)R * n_);
         // persistent sweep: spin-change ring, published fields, counters
         const bool blk = kernel_ == SG_SK_BLOCKED;
         pa_.Dring = c.take<uint8_t>(blk ? (size_t)kPersistSlots * R * 128 : 0);
@@ -653,6 +650,7 @@ private:
     std::vector<int32_t> h_tidx_;
     std::vector<float> h_coef_;
     SkDev d_{};
+    int8_t* d_spins_ = nullptr;  // the configuration as the caller reads it
     CUtensorMap mapJ_{}, mapD_{};
     int64_t *dC_ = nullptr, *dQ_ = nullptr, *dE_ = nullptr;
     int64_t *mC_ = nullptr, *mQ_ = nullptr, *mE_ = nullptr;

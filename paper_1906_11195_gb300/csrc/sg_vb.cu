@@ -253,6 +253,9 @@ public:
             std::vector<uint64_t> seeds(n_inst);
             for (int b = 0; b < n_inst; ++b) seeds[b] = graphs_[b].seed;
             up((void*)pk_.seeds, seeds.data(), seeds.size() * 8);
+            std::vector<int64_t> gw(1, 0);
+            for (const Graph& g : graphs_) gw.push_back(gw.back() + (int64_t)R * g.n);
+            up((void*)d_graph_words_, gw.data(), gw.size() * 8);
             up((void*)pk_.up_slice_base, h_up_base_.data(), h_up_base_.size() * 4);
             launches += vb_packed_build_upper(pk_, st);  // from col and jb, on the device
             launches += vb_packed_init(pk_, st);
@@ -541,17 +544,16 @@ public:
     void get_spins(void* dst, cudaStream_t st) override {
         uint64_t* out = static_cast<uint64_t*>(dst);
         if (kernel_ == SG_VB_PACKED) {
-            std::vector<uint64_t> S((size_t)pk_.n_slots * R);
-            down(S.data(), pk_.S, S.size() * 8, st);
-            check_cuda(cudaStreamSynchronize(st), "read spins");
-            int64_t off = 0;
-            for (int b = 0; b < n_inst; ++b) {
-                const Graph& g = graphs_[b];
-                for (int r = 0; r < R; ++r)
-                    for (int32_t v = 0; v < g.n; ++v)
-                        out[off + (int64_t)r * g.n + v] = S[(size_t)slot_of_[b][v] * R + r];
-                off += (int64_t)R * g.n;
+            // laid out in the caller's order on the device, a part at a time, and copied straight
+            // to the caller
+            const int64_t total = (int64_t)(spins_bytes() / 8);
+            for (int64_t lo = 0; lo < total; lo += spin_part()) {
+                const int64_t hi = std::min(total, lo + spin_part());
+                launches += vb_packed_spins(pk_, d_graph_words_, lo, hi, d_spins_, st);
+                check_cuda(cudaGetLastError(), "spins launch");
+                down(out + lo, d_spins_, (size_t)(hi - lo) * 8, st);
             }
+            check_cuda(cudaStreamSynchronize(st), "read spins");
         } else {
             const int32_t N = pl_.N;
             std::vector<int8_t> s((size_t)R * L * N);
@@ -607,6 +609,8 @@ public:
     }
 
 private:
+    // words of the configuration copied at a time (64 MB bounds the workspace for it)
+    int64_t spin_part() const { return std::min<int64_t>((int64_t)(spins_bytes() / 8), (int64_t)8 << 20); }
     size_t nC() const { return (size_t)n_inst * R * Lc_ * tw.size() * tm.size(); }
     size_t nQ() const { return (size_t)n_inst * (R / 2) * Lc_ * tm.size(); }
     size_t nE() const { return (size_t)n_inst * R * Lc_ * tm.size(); }
@@ -646,6 +650,8 @@ private:
             pk_.up_jb = c.take<uint64_t>(up_entries_);
             pk_.S = c.take<uint64_t>((size_t)n_slots_ * R);
             pk_.snap = c.take<uint64_t>((size_t)n_slots_ * R * tw.size());
+            d_spins_ = c.take<uint64_t>((size_t)spin_part());
+            d_graph_words_ = c.take<int64_t>((size_t)n_inst + 1);
             pk_.thr = d_thr_;
             pk_.n_slots = n_slots_;
             pk_.n_slices = (int32_t)(n_slots_ / 32);
@@ -909,6 +915,8 @@ private:
     VbPackedDev pk_{};
     VbPlainDev pl_{};
     uint32_t* d_thr_ = nullptr;
+    uint64_t* d_spins_ = nullptr;       // a part of the configuration in the caller's order
+    int64_t* d_graph_words_ = nullptr;  // [n_graphs + 1] first word of each graph in it
     int64_t *dC_ = nullptr, *dQ_ = nullptr, *dE_ = nullptr;
     int64_t *mC_ = nullptr, *mQ_ = nullptr, *mE_ = nullptr;
     int64_t *wC_ = nullptr, *wQ_ = nullptr, *wE_ = nullptr;  // window sums of raw counts

@@ -149,6 +149,8 @@ int sk_plain_sweep(const SkDev& d, const uint32_t* clock, uint32_t t_off, cudaSt
 int sk_measure(const SkDev& d, int n_active, int64_t* cdst, int64_t c_stride_r,
                int64_t c_stride_w, int64_t* qdst, int64_t q_stride_p, int64_t* edst,
                int64_t e_stride_r, cudaStream_t st);
+// the spins as int8 [R][N] (out 4-byte aligned)
+int sk_spins(const SkDev& d, int8_t* out, cudaStream_t st);
 int sk_snapshot(const SkDev& d, int w, cudaStream_t st);
 
 }  // namespace sg

@@ -622,6 +622,36 @@ int sk_measure(const SkDev& d, int n_active, int64_t* cdst, int64_t c_stride_r,
     return 1;
 }
 
+// The configuration as int8 [R][N] from the packed words: four consecutive outputs per thread.
+__global__ void k_sk_spins(SkDev d, int8_t* __restrict__ out) {
+    const int64_t total = (int64_t)d.R * d.N;
+    const int64_t k = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
+    if (k >= total) return;
+    const int words = d.Np / 32;
+    int r = (int)(k / d.N), i = (int)(k - (int64_t)r * d.N);
+    uint32_t v = 0;
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+        if (k + b < total && ((d.S[(int64_t)r * words + (i >> 5)] >> (i & 31)) & 1u)) v |= 0xFFu << (8 * b);
+        else v |= 1u << (8 * b);
+        if (++i == d.N) {
+            i = 0;
+            ++r;
+        }
+    }
+    if (k + 4 <= total) {
+        *reinterpret_cast<uint32_t*>(out + k) = v;
+    } else {
+        for (int b = 0; k + b < total; ++b) out[k + b] = (int8_t)(v >> (8 * b));
+    }
+}
+
+int sk_spins(const SkDev& d, int8_t* out, cudaStream_t st) {
+    const int64_t n = ((int64_t)d.R * d.N + 3) / 4;
+    k_sk_spins<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(d, out);
+    return 1;
+}
+
 __global__ void k_copy_words(const uint4* __restrict__ src, uint4* __restrict__ dst, int64_t n16) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n16;
          i += (int64_t)gridDim.x * blockDim.x)
