@@ -118,11 +118,11 @@ def peaks():
 
 
 def kernel_source_hash():
-    """Hash of the colour kernel's code (comments and layout removed, so a comment edit does
+    """Hash of the sweep kernel's code (comments and layout removed, so a comment edit does
     not invalidate the recorded traffic, while any code change does)."""
     import re
     h = hashlib.sha256()
-    for f in ("vb_colour.cuh", "sg_internal.cuh"):
+    for f in ("vb_sweep.cu", "vb_bits.cuh", "sg_internal.cuh"):
         with open(os.path.join(ROOT, "paper_1906_11195_gb300", "csrc", f)) as fh:
             src = fh.read()
         src = re.sub(r"/\*.*?\*/", " ", src, flags=re.S)
@@ -132,7 +132,7 @@ def kernel_source_hash():
 
 
 def recorded_traffic():
-    """DRAM bytes per sweep of the colour kernel from the committed ncu summary, if it was
+    """DRAM bytes per sweep of the sweep kernel from the committed ncu summary, if it was
     taken on the current kernel source."""
     p = os.path.join(ROOT, "profiles", "vb_packed_colour_traffic.json")
     if not os.path.exists(p):
@@ -382,7 +382,7 @@ def run_reference(args):
 
 def run_profile_case(args):
     """One T = 1.0 instance of the full-size graph with no measurement schedule: W + K sweeps.
-    This is the small case used for detailed ncu captures of the colour kernel (about 0.3 GB on
+    This is the small case used for detailed ncu captures of the sweep kernel (about 0.3 GB on
     the device, inputs larger than L2).  With --workload sk: the SK workload's handle (N = 8192,
     256 replicas, T = 0.4, B = 128, about 0.4 GB on the device), W sweeps and then K sweeps in
     one call (one persistent launch per replayed graph).  Prints timing only; not a bench line."""
@@ -632,7 +632,7 @@ def measure_vb_batch(args, dev, stream, steps, warmup, cpu=True, count=512):
                       "l2": f"inputs larger than L2: {bytes_sweep / 1e9:.2f} GB streamed per sweep"},
            "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                         "frac": achieved / peak, "traffic": None, "peak_source": peak_kind,
-                        "kernel": "k_vb_packed_colour over the whole batch, one unit = one sweep",
+                        "kernel": "k_vb_sweeps over the whole batch, one unit = one sweep",
                         "algorithmic_bytes_per_sweep": bytes_sweep,
                         "note": "achieved over the timed region (measurements included)"},
            "clocks": clocks}
@@ -1074,7 +1074,7 @@ def run_gpu(args):
     for r in runs:
         r.close()
 
-    # roofline of the colour kernel: a handle with no measurement schedule times pure sweeps
+    # roofline of the sweep kernel: a handle with no measurement schedule times pure sweeps
     kr = max(20, min(args.steps, 200))
     rl = sg.VBRun([graphs[0]], n_lanes=LANES, n_replicas=REPLICAS, kernel=sg.SG_VB_PACKED,
                   device=dev, stream=stream)
@@ -1089,7 +1089,7 @@ def run_gpu(args):
     rl.close()
     bytes_sweep = algorithmic_bytes_per_sweep(N_VERTS, int(rp[-1]), REPLICAS)
     peak, peak_kind = peaks()
-    # achieved: the colour kernel's algorithmic bytes of every sweep in the timed region over the
+    # achieved: the sweep kernel's algorithmic bytes of every sweep in the timed region over the
     # whole timed region (the few snapshot/measurement launches in it count against the kernel,
     # so this is a lower bound); achieved_isolated: the same over sweeps timed alone
     sweep_ms_timed = ms / (args.steps * len(TEMPS))
@@ -1097,12 +1097,12 @@ def run_gpu(args):
     traffic = recorded_traffic()
     roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                 "frac": achieved / peak, "traffic": traffic, "peak_source": peak_kind,
-                "kernel": "k_vb_packed_colour<2>, one unit = one sweep (all colour classes)",
+                "kernel": "k_vb_sweeps<2>, one unit = one sweep (all colour classes)",
                 "algorithmic_bytes_per_sweep": bytes_sweep, "ms_per_sweep": sweep_ms_timed,
                 "achieved_isolated": bytes_sweep / (sweep_ms * 1e-3) / 1e9,
                 "ms_per_sweep_isolated": sweep_ms,
                 "frac_kernel": bytes_sweep / (sweep_ms * 1e-3) / 1e9 / peak,
-                "note": "frac: the colour kernel's algorithmic bytes over the whole timed step "
+                "note": "frac: the sweep kernel's algorithmic bytes over the whole timed step "
                         "(snapshot and measurement launches included); frac_kernel: the same "
                         "over sweeps timed alone (no schedule), the kernel's own fraction; "
                         "traffic: DRAM bytes per sweep from the committed ncu summary of this "
@@ -1162,7 +1162,7 @@ def run_gpu(args):
            "phases": phases,
            "note": "H2D of both instances' images at attach + sweeps + D2H of all counts (bytes "
                    "counted by the library), spread over the steps; phases: host time of the "
-                   "attach calls (copies, autotuner), the sweep calls (queued) and the reads "
+                   "attach calls (copies), the sweep calls (queued) and the reads "
                    "(which wait for the sweeps)"}
 
     # the other configurations of the metric, each with its own value, roofline, e2e, clocks

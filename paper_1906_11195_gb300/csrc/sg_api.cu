@@ -131,6 +131,7 @@ static cudaGraphExec_t sweep_graph(sg_handle h, int k) {
 static void run_sweeps(sg_handle h, int64_t t0, int64_t len) {
     if (len <= 0) return;
     sg::Model& m = *h->model;
+    if (m.sweep_direct(t0, len, h->stream)) return;
     sg::k_clock_set<<<1, 1, 0, h->stream>>>(m.clock_dev, (uint32_t)t0);
     m.launches += 1;
     if (h->max_graph_log < 0) {

@@ -168,13 +168,9 @@ struct VbPackedDev {
     const uint64_t* jb;          // [n_entries] coupling word (0 for padding entries)
     const uint64_t* seeds;       // [n_graphs]
     const uint32_t* thr;         // [n_graphs][R][64]
-    const uint4* groups;         // [n_groups] {first slice, slices, first entry, entries}
     const uint4* slice_meta;     // [n_slices] {first entry, width, graph, 0}
-    const uint32_t* group_graph; // [n_groups] graph of each group (groups never mix graphs)
-    const uint8_t* gtab;         // [n_graphs] {uint32 thr[R][64]; uint64 seed; uint64 pad}
-    const uint32_t* colour_groups;  // [n_colours+1] first group of each colour class
     int* err;                    // device status word (bounded waits)
-    uint32_t* gbar;              // [2] grid-barrier arrivals and exits of a fused sweep (zeroed)
+    uint32_t* gbar;              // [2] grid-barrier arrivals and exits of a sweep launch (zeroed)
     uint64_t* S;                 // [n_slots][R]
     uint64_t* snap;              // [n_tw][n_slots][R]
     // upper entries for the energy: per slice, each lane's neighbours in later colour classes
@@ -189,7 +185,9 @@ struct VbPackedDev {
     int32_t R;
     int32_t n_colours;
     int32_t n_graphs;
-    uint64_t stage_wait_ns;      // bound of one pipeline wait in the colour kernel
+    const uint32_t* class_slice; // [n_colours+1] first slice of each colour class
+    bool stream_first;           // the graph does not fit L2 beside the spins: its lines leave first
+    uint64_t stage_wait_ns;      // bound of one wait at the sweeps' grid barrier
 };
 
 constexpr int kVbMaxColours = 64;  // greedy colouring with degree <= 63
@@ -232,16 +230,11 @@ struct VbMeasure {
 
 // launch wrappers (vb_kernels.cu); each returns the number of kernel launches queued
 int vb_packed_init(const VbPackedDev& d, cudaStream_t st);
-// sweep index t = *clock + t_off (the clock lives in device memory so that captured CUDA graphs
-// can be replayed at any time)
-// One sweep of every colour class in colour order.  variant (0 .. kVbColourVariants - 1)
-// selects the pipeline shape (stream stages, gather buffers, gather lookahead, CTAs per SM);
-// fused runs the classes in one cooperative launch with grid-wide barriers between them
-// (R = 2, 4), else one launch per class.  colour_groups is the host copy of d.colour_groups.
-// No choice changes the results.  Returns the launches queued, or -1.
-int vb_packed_sweep(const VbPackedDev& d, const uint32_t* colour_groups, const uint32_t* clock,
-                    uint32_t t_off, int variant, bool fused, cudaStream_t st);
-constexpr int kVbColourVariants = 3;
+// n sweeps with indices t0, t0 + 1, ..., every colour class in colour order, in one cooperative
+// launch (vb_sweep.cu); max_class_slices: slices of the largest class.  Returns the launches
+// queued, or -1.
+int vb_packed_sweeps(const VbPackedDev& d, int max_class_slices, uint32_t t0, int n_sweeps,
+                     cudaStream_t st);
 // words [lo, hi) of the configuration in the caller's order (graph_words: first word of each graph)
 int vb_packed_spins(const VbPackedDev& d, const int64_t* graph_words, int64_t lo, int64_t hi,
                     uint64_t* out, cudaStream_t st);
@@ -253,6 +246,8 @@ int vb_packed_build_upper(const VbPackedDev& d, cudaStream_t st);
 int vb_packed_measure(const VbPackedDev& d, const VbMeasure& m, cudaStream_t st);
 
 int vb_plain_init(const VbPlainDev& d, cudaStream_t st);
+// sweep index t = *clock + t_off (the clock lives in device memory so that captured CUDA graphs
+// can be replayed at any time)
 int vb_plain_colour(const VbPlainDev& d, int32_t v_begin, int32_t v_end, const uint32_t* clock,
                     uint32_t t_off, cudaStream_t st);
 int vb_plain_snapshot(const VbPlainDev& d, int w, cudaStream_t st);

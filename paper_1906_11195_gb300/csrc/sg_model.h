@@ -87,6 +87,14 @@ public:
     virtual void sweep_many(uint32_t t_off, int n, cudaStream_t st) {
         for (int s = 0; s < n; ++s) sweep(t_off + (uint32_t)s, st);
     }
+    // n consecutive sweeps from time t0 queued without a captured graph, if the model has a launch
+    // that takes them all; false: not done
+    virtual bool sweep_direct(int64_t t0, int64_t n, cudaStream_t st) {
+        (void)t0;
+        (void)n;
+        (void)st;
+        return false;
+    }
     // snapshot w <- current spins
     virtual void snapshot(int w, cudaStream_t st) = 0;
     // scheduled measurement column u at time tau (snapshots with tw <= tau exist)

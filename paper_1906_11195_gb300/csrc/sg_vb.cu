@@ -14,9 +14,7 @@
 
 #include <algorithm>
 #include <atomic>
-#include <map>
 #include <memory>
-#include <mutex>
 #include <string>
 #include <thread>
 #include <vector>
@@ -242,13 +240,10 @@ public:
             up((void*)pk_.slice_base, h_slice_base_.data(), h_slice_base_.size() * 4);
             up((void*)pk_.slice_graph, h_slice_graph_.data(), h_slice_graph_.size() * 4);
             up((void*)pk_.col, h_col_.data(), h_col_.size() * 4);
-            up((void*)pk_.groups, h_groups_.data(), h_groups_.size() * sizeof(uint4));
             up((void*)pk_.slice_meta, h_slice_meta_.data(), h_slice_meta_.size() * sizeof(uint4));
-            up((void*)pk_.group_graph, h_group_graph_.data(), h_group_graph_.size() * 4);
-            up((void*)pk_.gtab, h_gtab_.data(), h_gtab_.size());
             check_cuda(cudaMemsetAsync(pk_.err, 0, 4, st), "memset");
-            up((void*)pk_.colour_groups, colour_group_.data(), colour_group_.size() * 4);
             check_cuda(cudaMemsetAsync(pk_.gbar, 0, 8, st), "memset");
+            up((void*)pk_.class_slice, colour_slice_.data(), colour_slice_.size() * 4);
             up((void*)pk_.jb, h_jb_.data(), h_jb_.size() * 8);
             std::vector<uint64_t> seeds(n_inst);
             for (int b = 0; b < n_inst; ++b) seeds[b] = graphs_[b].seed;
@@ -259,21 +254,6 @@ public:
             up((void*)pk_.up_slice_base, h_up_base_.data(), h_up_base_.size() * 4);
             launches += vb_packed_build_upper(pk_, st);  // from col and jb, on the device
             launches += vb_packed_init(pk_, st);
-            // SG_VB_COLOUR_VARIANT=<k> and SG_VB_FUSED=<0|1> pin the pipeline shape and the
-            // launch form (reproducible timings of one choice); otherwise the autotuner picks
-            const char* pin = getenv("SG_VB_COLOUR_VARIANT");
-            const char* pin_f = getenv("SG_VB_FUSED");
-            const bool pinned = pin && *pin >= '0' && *pin < '0' + kVbColourVariants && !pin[1];
-            const bool pinned_f = pin_f && (*pin_f == '0' || *pin_f == '1') && !pin_f[1];
-            if (pinned && pinned_f) {
-                variant_ = *pin - '0';
-                fused_ = *pin_f == '1';
-            } else if (!pinned && !pinned_f && tuned_before()) {
-                // an instance of the same layout was tuned in this process: its choice holds
-            } else {
-                tune_variant(st, pinned ? *pin - '0' : -1, pinned_f ? *pin_f - '0' : -1);
-                if (!pinned && !pinned_f) remember_tuning();
-            }
         } else {
             up((void*)pl_.row_ptr, h_row_ptr_.data(), h_row_ptr_.size() * 4);
             up((void*)pl_.col, h_col_i_.data(), h_col_i_.size() * 4);
@@ -293,101 +273,26 @@ public:
         check_cuda(cudaStreamSynchronize(st), "attach");
     }
 
-    // The autotuner's choice per layout shape (slots, entries, colour classes, groups, replicas,
-    // device), kept for the process: the timings depend on nothing else.
-    using TuneKey = std::vector<int64_t>;
-    static std::mutex& tune_mutex() {
-        static std::mutex m;
-        return m;
-    }
-    static std::map<TuneKey, std::pair<int, bool>>& tune_cache() {
-        static std::map<TuneKey, std::pair<int, bool>> c;
-        return c;
-    }
-    TuneKey tune_key() const {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        TuneKey k{dev, n_slots_, (int64_t)h_col_.size(), (int64_t)colour_group_.size(),
-                  (int64_t)h_groups_.size(), R, n_inst};
-        k.insert(k.end(), colour_group_.begin(), colour_group_.end());
-        return k;
-    }
-    bool tuned_before() {
-        std::lock_guard<std::mutex> g(tune_mutex());
-        auto it = tune_cache().find(tune_key());
-        if (it == tune_cache().end()) return false;
-        variant_ = it->second.first;
-        fused_ = it->second.second;
-        return true;
-    }
-    void remember_tuning() {
-        std::lock_guard<std::mutex> g(tune_mutex());
-        tune_cache()[tune_key()] = {variant_, fused_};
-    }
-
-    // Autotuner: time two sweeps with each pipeline shape of the colour kernel, launched per
-    // colour class and (R = 2, 4) fused into one cooperative launch per sweep, and keep the
-    // fastest; then redraw the initial spins (the trial sweeps leave no trace: the initial
-    // configuration is a pure function of the seed, and no measurement was taken).  A choice
-    // whose launch is refused (e.g. a cooperative grid that cannot be resident) is skipped.
-    // only_v / only_f >= 0 restrict the search to one shape / launch form.
-    void tune_variant(cudaStream_t st, int only_v, int only_f) {
-        cudaEvent_t e0, e1;
-        check_cuda(cudaEventCreate(&e0), "cudaEventCreate");
-        check_cuda(cudaEventCreate(&e1), "cudaEventCreate");
-        float best = 0.f;
-        int best_v = -1;
-        bool best_f = false;
-        const bool can_fuse = R != 1 && colour_group_.size() > 2;
-        if (!can_fuse) only_f = -1;  // a fused request runs per class (as the sweep does)
-        for (int f = 0; f < (can_fuse ? 2 : 1); ++f) {
-            if (only_f >= 0 && f != only_f) continue;
-            for (int v = 0; v < kVbColourVariants; ++v) {
-                if (only_v >= 0 && v != only_v) continue;
-                variant_ = v;
-                fused_ = f == 1;
-                float ms = 0.f;
-                try {
-                    check_cuda(cudaMemsetAsync(clock_dev, 0, 4, st), "memset");
-                    sweep(0, st);  // warm-up
-                    check_cuda(cudaEventRecord(e0, st), "cudaEventRecord");
-                    sweep(1, st);
-                    sweep(2, st);
-                    check_cuda(cudaEventRecord(e1, st), "cudaEventRecord");
-                    check_cuda(cudaEventSynchronize(e1), "cudaEventSynchronize");
-                    check_cuda(cudaEventElapsedTime(&ms, e0, e1), "cudaEventElapsedTime");
-                } catch (const Error&) {
-                    cudaGetLastError();
-                    check_cuda(cudaStreamSynchronize(st), "autotuner");
-                    continue;
-                }
-                if (best_v < 0 || ms < best) {
-                    best = ms;
-                    best_v = v;
-                    best_f = fused_;
-                }
-            }
+    // The packed sweeps of a call, without a captured graph: a launch takes as many sweeps as run in a few
+    // milliseconds, so nothing is left of the launches' gaps.
+    bool sweep_direct(int64_t t0, int64_t n, cudaStream_t st) override {
+        if (kernel_ != SG_VB_PACKED) return false;
+        const int64_t most = std::max<int64_t>(1, std::min<int64_t>(1024, ((int64_t)1 << 28) / (n_slots_ * R)));
+        for (int64_t done = 0; done < n;) {
+            const int m = (int)std::min<int64_t>(n - done, most);
+            const uint32_t t = (uint32_t)(t0 + done);
+            const int k = vb_packed_sweeps(pk_, max_class_slices_, t, m, st);
+            if (k < 0) fail(SG_ECUDA, "sweep launch failed");
+            launches += k;
+            done += m;
         }
-        cudaEventDestroy(e0);
-        cudaEventDestroy(e1);
-        if (best_v < 0) fail(SG_ECUDA, "no colour-kernel configuration could be launched");
-        if (device_status(st)) fail(SG_ETIMEOUT, "device wait expired while tuning the colour kernel");
-        variant_ = best_v;
-        fused_ = best_f;
-        launches += vb_packed_init(pk_, st);
+        return true;
     }
 
     void sweep(uint32_t t_off, cudaStream_t st) override {
-        if (kernel_ == SG_VB_PACKED) {
-            const int n = vb_packed_sweep(pk_, colour_group_.data(), clock_dev, t_off, variant_,
-                                          fused_, st);
-            if (n < 0) fail(SG_ECUDA, "colour kernel launch failed");
-            launches += n;
-        } else {
-            for (size_t c = 0; c + 1 < colour_begin_.size(); ++c)
-                launches += vb_plain_colour(pl_, colour_begin_[c], colour_begin_[c + 1], clock_dev,
-                                            t_off, st);
-        }
+        if (kernel_ == SG_VB_PACKED) fail(SG_EINVAL, "packed sweeps are queued by sweep_direct");
+        for (size_t c = 0; c + 1 < colour_begin_.size(); ++c)
+            launches += vb_plain_colour(pl_, colour_begin_[c], colour_begin_[c + 1], clock_dev, t_off, st);
     }
 
     void snapshot(int w, cudaStream_t st) override {
@@ -634,13 +539,12 @@ private:
             pk_.slice_base = c.take<uint32_t>(h_slice_base_.size());
             pk_.slice_graph = c.take<uint32_t>(h_slice_graph_.size());
             pk_.col = c.take<uint32_t>(h_col_.size());
-            pk_.groups = c.take<uint4>(h_groups_.size());
             pk_.slice_meta = c.take<uint4>(h_slice_meta_.size());
-            pk_.group_graph = c.take<uint32_t>(h_group_graph_.size());
-            pk_.gtab = c.take<uint8_t>(h_gtab_.size());
             pk_.err = c.take<int>(1);
-            pk_.colour_groups = c.take<uint32_t>(colour_group_.size());
             pk_.gbar = c.take<uint32_t>(2);
+            pk_.class_slice = c.take<uint32_t>(colour_slice_.size());
+            // about 96 MB of the 129 MB L2 for graph and spins together
+            pk_.stream_first = h_col_.size() * 12 + (size_t)n_slots_ * (4 + 8 * R) > ((size_t)96 << 20);
             pk_.jb = c.take<uint64_t>(h_jb_.size());
             pk_.seeds = c.take<uint64_t>(n_inst);
             pk_.up_slice_base = c.take<uint32_t>(h_up_base_.size());
@@ -657,7 +561,7 @@ private:
             pk_.n_slices = (int32_t)(n_slots_ / 32);
             pk_.R = R;
             pk_.n_graphs = n_inst;
-            pk_.n_colours = (int32_t)colour_group_.size() - 1;
+            pk_.n_colours = (int32_t)colour_slice_.size() - 1;
             // SG_TEST_STAGE_WAIT_NS shortens the colour kernel's pipeline waits: a test of the
             // timeout path (the kernel gives up, flags SG_ETIMEOUT and exits cleanly)
             pk_.stage_wait_ns = 2000000000ull;
@@ -762,6 +666,8 @@ private:
             }
         }
         colour_slice_[cmax] = (uint32_t)(cursor / 32);
+        for (int c = 0; c < cmax; ++c)
+            max_class_slices_ = std::max(max_class_slices_, (int)(colour_slice_[c + 1] - colour_slice_[c]));
         n_slots_ = cursor;
         const int64_t n_slices = n_slots_ / 32;
         h_vinfo_.assign(n_slots_, kInactive);
@@ -852,55 +758,17 @@ private:
             m.w = 0;
             h_slice_meta_[s] = m;
         }
-        // staging groups: consecutive slices of one colour, <= 8 slices and <= 1024 entries;
-        // a single slice wider than that (degree > 32) forms a group flagged "wide"
-        colour_group_.assign(cmax + 1, 0);
-        for (int c = 0; c < cmax; ++c) {
-            colour_group_[c] = (uint32_t)h_groups_.size();
-            int64_t s = colour_slice_[c];
-            while (s < (int64_t)colour_slice_[c + 1]) {
-                const int64_t first = s;
-                while (s < (int64_t)colour_slice_[c + 1] && s - first < 8 &&
-                       h_slice_graph_[s] == h_slice_graph_[first] &&
-                       (int64_t)h_slice_base_[s + 1] - (int64_t)h_slice_base_[first] <= 1024)
-                    ++s;
-                bool wide = false;
-                if (s == first) {  // one slice alone exceeds the stage
-                    ++s;
-                    wide = true;
-                }
-                uint4 gi;
-                gi.x = (uint32_t)first;
-                gi.y = (uint32_t)(s - first) | (wide ? 0x80000000u : 0u);
-                gi.z = h_slice_base_[first];
-                gi.w = h_slice_base_[s] - h_slice_base_[first];
-                h_groups_.push_back(gi);
-                h_group_graph_.push_back(h_slice_graph_[first]);
-            }
-        }
-        // per-graph table staged with each group: thresholds of the R replicas, then the key
-        const size_t gtab_bytes = (size_t)R * kVbThrStride * 4 + 16;
-        h_gtab_.assign(gtab_bytes * n_inst, 0);
-        for (int b = 0; b < n_inst; ++b) {
-            memcpy(&h_gtab_[b * gtab_bytes], &thr_[(size_t)b * R * kVbThrStride],
-                   (size_t)R * kVbThrStride * 4);
-            memcpy(&h_gtab_[b * gtab_bytes + (size_t)R * kVbThrStride * 4], &graphs_[b].seed, 8);
-        }
-        colour_group_[cmax] = (uint32_t)h_groups_.size();
     }
 
     int kernel_ = SG_VB_PACKED;
-    int variant_ = 0;     // colour-kernel pipeline shape chosen by the autotuner at attach
-    bool fused_ = false;  // one cooperative launch per sweep (else one launch per colour class)
+    int max_class_slices_ = 0;  // slices of the largest class
     int Lc_ = 64;
     size_t ws_bytes_ = 0;
     std::vector<Graph> graphs_;
     std::vector<uint32_t> thr_;
     // packed host layout
-    std::vector<uint32_t> colour_slice_, colour_group_;
-    std::vector<uint4> h_groups_, h_slice_meta_;
-    std::vector<uint32_t> h_group_graph_;
-    std::vector<uint8_t> h_gtab_;
+    std::vector<uint32_t> colour_slice_;
+    std::vector<uint4> h_slice_meta_;
     std::vector<std::vector<int64_t>> slot_of_;
     int64_t n_slots_ = 0;
     std::vector<uint32_t> h_slice_base_, h_slice_graph_;

@@ -91,6 +91,22 @@ __device__ __forceinline__ void half_add(uint64_t a, uint64_t b, uint64_t& s, ui
     cy = a & b;
 }
 
+// p += x0 + x1 + x2 + x3, lane by lane (the sum fits P planes)
+template <int P>
+__device__ __forceinline__ void bitslice_add4(uint64_t (&p)[P], uint64_t x0, uint64_t x1, uint64_t x2,
+                                              uint64_t x3) {
+    uint64_t c1, c2, c;
+    full_add(p[0], x0, x1, p[0], c1);
+    full_add(p[0], x2, x3, p[0], c2);
+    full_add(p[1], c1, c2, p[1], c);
+#pragma unroll
+    for (int b = 2; b < P; ++b) {
+        const uint64_t s = p[b] ^ c;
+        c = p[b] & c;
+        p[b] = s;
+    }
+}
+
 // planes needed to count W one-bit inputs
 template <int W>
 struct CountBits { static constexpr int P = W <= 1 ? 1 : W <= 3 ? 2 : W <= 7 ? 3 : 4; };

@@ -1,5 +1,5 @@
-// vb_kernels.cu -- Viana-Bray Metropolis kernels for sm_103a (the colour-class sweep itself is
-// in vb_colour.cuh).
+// vb_kernels.cu -- Viana-Bray Metropolis kernels for sm_103a (the packed sweeps are in
+// vb_sweep.cu and vb_resident.cu).
 //
 // Model (Eq. 3): H = -sum_{(ij) in E} J_ij s_i s_j, J_ij = +-1.  Flipping s_i changes the
 // energy by dE = 2m with m = s_i sum_j J_ij s_j = d_i - 2u_i, u_i the number of unsatisfied
@@ -10,12 +10,13 @@
 // Packed kernel (multispin coding, SI section 2): bit k of a uint64 spin word is lane k (an
 // independent disorder sample); one thread updates one vertex for all 64 lanes and all R
 // replicas.  Per neighbour, x = S_i ^ S_j ^ J marks the unsatisfied lanes; the x words are
-// summed into a bit-sliced count (an unrolled carry-save adder tree for slices of width <= 8,
-// a ripple counter of up to 6 planes, degree <= 63, otherwise).  Because thr[m] is
+// summed into a bit-sliced count (carry-save adders, four words at a time, up to width 15; a
+// ripple counter of 6 planes, degree <= 63, beyond).  Because thr[m] is
 // non-increasing in m and the random number is shared by the 64 lanes, the accepted set
 // {m <= m*} is a prefix: with m* = #{m in 1..d : r32 < thr[m]}, a lane flips iff d - 2u <= m*,
 // i.e. u >= ceil((d - m*)/2): one bit-sliced compare against a per-thread constant.
-#include "vb_colour.cuh"
+#include "../../include/sg.h"
+#include "sg_internal.cuh"
 
 namespace sg {
 

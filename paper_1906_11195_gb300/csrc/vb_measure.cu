@@ -31,22 +31,6 @@ struct MeasureGrid {
     uint32_t up_rows;
 };
 
-// p += x0 + x1 + x2 + x3, lane by lane
-template <int P>
-__device__ __forceinline__ void add4(uint64_t (&p)[P], uint64_t x0, uint64_t x1, uint64_t x2,
-                                     uint64_t x3) {
-    uint64_t c1, c2, c;
-    full_add(p[0], x0, x1, p[0], c1);
-    full_add(p[0], x2, x3, p[0], c2);
-    full_add(p[1], c1, c2, p[1], c);
-#pragma unroll
-    for (int b = 2; b < P; ++b) {
-        const uint64_t s = p[b] ^ c;
-        c = p[b] & c;
-        p[b] = s;
-    }
-}
-
 // Sum the counters of the warp's 32 threads.  The first exchange leaves each half warp with one
 // 32-bit half of the words, the others add within the half warp, one more plane each; thread l
 // then holds the totals of lanes 32 (l / 16) + l % 16 (c0) and 16 above it (c1).
@@ -139,7 +123,7 @@ __device__ __forceinline__ void count_rows(const VbPackedDev& d, const uint64_t*
 #pragma unroll
         for (int u = 0; u < 4; ++u) row(s + u, s + u < b, x[u]);
 #pragma unroll
-        for (int q = 0; q < NQ; ++q) add4(p[q], x[0][q], x[1][q], x[2][q], x[3][q]);
+        for (int q = 0; q < NQ; ++q) bitslice_add4(p[q], x[0][q], x[1][q], x[2][q], x[3][q]);
     }
 }
 

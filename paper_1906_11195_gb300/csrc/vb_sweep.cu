@@ -1,0 +1,386 @@
+// vb_sweep.cu -- the packed Viana-Bray sweep for sm_103a: several sweeps in one cooperative launch,
+// one thread per vertex for all 64 lanes and all R replicas (multispin coding, SI section 2), one
+// colour class (an independent set) at a time, the generalisation of the bipartite half-updates of
+// SI section 3, with a grid-wide barrier between classes.
+//
+// A warp owns the same slices (32 vertices of one class, degree-sorted) in every sweep.  Its work is
+// a chain of chunks of four (or eight) sliced-ELL entries: while the neighbours' words of one chunk are on
+// their way from L2, the neighbour slots and coupling words of the next chunk (of the next slice,
+// the next class or the next sweep: nothing a sweep writes, except a vertex's own words, which only
+// this thread writes) are already being read into registers, and the next slice's random numbers
+// and acceptance thresholds are worked out before the barrier that admits its gathers.
+//
+// What bounds it.  Small and middling graphs: a class takes about 2.3 us of latencies (the stores'
+// release, the barrier's way through L2 and back, a gather) before any work.  Large ones: a sweep
+// of N = 2^22 (degree 4, two replicas) reads 84 bytes per vertex from HBM (31 % of its peak), gathers
+// 16.8 million word pairs, each a 32-byte sector of L2 (45 %) and a tag of L1 (50 %), and issues 515
+// instructions per slice (41 %).  us a sweep, before (groups staged by bulk copies into shared-memory
+// rings, a launch per sweep) -> now: N = 2^22 131 -> 128, 2^20 50 -> 39, bipartite 2^18 14.2 -> 10.3,
+// N = 300007 with one replica (a launch per class) 30.8 -> 17, N = 20011 with four 23.3 -> 18.3.
+// Without the rings there is no pipeline to fill and drain in each class, and no launch gap.
+#include <algorithm>
+
+#include "../../include/sg.h"
+#include "sg_internal.cuh"
+#include "vb_bits.cuh"
+
+namespace sg {
+
+namespace {
+
+// threads of a CTA (two CTAs share an SM) and entries per chunk
+template <int R, int CH>
+struct SweepShape {
+    static constexpr int threads = CH == 8 ? (R == 4 ? 192 : 256) : R == 1 ? 384 : R == 2 ? 320 : 256;
+};
+
+constexpr int kSweepTables = 16;  // graphs whose thresholds are kept in shared memory
+constexpr int kSweepPlanes = 4;  // counter planes: slices up to width 15; wider ones count apart
+
+__device__ __forceinline__ uint32_t ld_stream_u32(const uint32_t* p, uint64_t pol) {
+    uint32_t v;
+    asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.u32 %0, [%1], %2;"
+                 : "=r"(v) : "l"(p), "l"(pol));
+    return v;
+}
+__device__ __forceinline__ uint64_t ld_stream_u64(const uint64_t* p, uint64_t pol) {
+    uint64_t v;
+    asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.u64 %0, [%1], %2;"
+                 : "=l"(v) : "l"(p), "l"(pol));
+    return v;
+}
+
+// spin words through L2 only: other CTAs write them within the launch
+template <int R>
+__device__ __forceinline__ SpinWords<R> ld_spins(const uint64_t* p, uint64_t pol) {
+    SpinWords<R> s;
+    if constexpr (R == 1) {
+        asm volatile("ld.global.cg.L2::cache_hint.u64 %0, [%1], %2;" : "=l"(s.v[0]) : "l"(p), "l"(pol) : "memory");
+    } else {
+#pragma unroll
+        for (int h = 0; h < R / 2; ++h)
+            asm volatile("ld.global.cg.L2::cache_hint.v2.u64 {%0, %1}, [%2], %3;"
+                         : "=l"(s.v[2 * h]), "=l"(s.v[2 * h + 1]) : "l"(p + 2 * h), "l"(pol) : "memory");
+    }
+    return s;
+}
+
+// Acceptance of one vertex: one Philox block per (vertex, sweep) serves replicas 0..3; the accepted
+// m form a prefix 1..m*, so a lane flips iff its unsatisfied count u reaches ceil((d - m*) / 2).
+// The first three thresholds come in one load (thr: shared or global memory); few draws pass all
+// three.
+template <int R>
+__device__ __forceinline__ void accept_from(uint32_t vi, uint32_t t, uint64_t seed,
+                                            const uint32_t* thr, int (&kmin)[R]) {
+    const int deg = vi == kInactive ? 0 : (int)(vi >> kDegShift);
+    const uint4 rnd = philox4x32_10(make_uint4(vi & kOrigMask, t, 0u, 0u), (uint32_t)seed,
+                                    (uint32_t)(seed >> 32));
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const uint32_t r32 = uint4_word(rnd, r);
+        const uint4 th = *reinterpret_cast<const uint4*>(thr + r * kVbThrStride);
+        int ms = (int)(r32 < th.y) + (int)(r32 < th.z) + (int)(r32 < th.w);
+        if (ms == 3)
+            while (ms < deg && r32 < thr[r * kVbThrStride + ms + 1]) ++ms;
+        ms = ms < deg ? ms : deg;
+        kmin[r] = (deg - ms + 1) >> 1;
+    }
+}
+
+__device__ __forceinline__ uint32_t ld_relaxed_u32(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+// the position of a warp in the sequence (sweep, class, slice)
+struct Cursor {
+    uint32_t sweep, cls, slice;
+};
+
+}  // namespace
+
+template <int R, int kChunk>
+__global__ void __launch_bounds__(SweepShape<R, kChunk>::threads, 2)
+    k_vb_sweeps(VbPackedDev d, uint32_t t0, uint32_t n_sweeps) {
+    __shared__ uint32_t cs[kVbMaxColours + 1];  // first slice of each class
+    __shared__ int s_ok;
+    __shared__ __align__(16) uint32_t s_thr[kSweepTables * R * kVbThrStride];
+    __shared__ uint64_t s_seed[kSweepTables];
+    const uint32_t tid = threadIdx.x, lane = tid & 31u;
+    const uint32_t nc = (uint32_t)d.n_colours;
+    const uint32_t gw = (tid >> 5) * gridDim.x + blockIdx.x;  // neighbouring slices on different SMs
+    const uint32_t stride = (blockDim.x >> 5) * gridDim.x;  // at least a CTA's warps: one round in the tail
+    for (uint32_t i = tid; i <= nc; i += blockDim.x) cs[i] = __ldg(d.class_slice + i);
+    const bool tables = d.n_graphs <= kSweepTables;
+    if (tables) {
+        for (uint32_t i = tid; i < (uint32_t)(d.n_graphs * R * kVbThrStride); i += blockDim.x) s_thr[i] = __ldg(d.thr + i);
+        for (uint32_t i = tid; i < (uint32_t)d.n_graphs; i += blockDim.x) s_seed[i] = __ldg(d.seeds + i);
+    }
+    if (tid == 0) s_ok = 1;
+    __syncthreads();
+    const uint32_t* thr = tables ? s_thr : d.thr;
+    const uint64_t* seeds = tables ? s_seed : d.seeds;
+    const uint64_t pol_keep = l2_evict_last();
+    const uint64_t pol_stream = d.stream_first ? l2_evict_first() : pol_keep;
+
+    // move to the warp's next slice, if there is one (sweep == n_sweeps: none)
+    // the thin classes at the end, each at most one slice per warp of a CTA, are all the first CTA's:
+    // they need no grid-wide barrier between them
+    const uint32_t warps = blockDim.x >> 5;
+    uint32_t tail = nc;
+    while (tail > 0 && cs[tail] - cs[tail - 1] <= warps) --tail;
+    auto first_slice = [&](uint32_t cls) -> uint32_t {
+        return cs[cls] + (cls < tail ? gw : blockIdx.x == 0 ? tid >> 5 : warps);
+    };
+    auto settle = [&](Cursor& c) {
+        while (c.sweep < n_sweeps && c.slice >= cs[c.cls + 1]) {
+            if (++c.cls == nc) {
+                c.cls = 0;
+                ++c.sweep;
+            }
+            c.slice = first_slice(c.cls);
+        }
+    };
+    auto load_meta = [&](const Cursor& c) -> uint4 {
+        return c.sweep < n_sweeps ? __ldg(d.slice_meta + c.slice) : make_uint4(0u, 0u, 0u, 0u);
+    };
+
+    // the next slice: position, {first entry, width, graph}, label and degree, own words, the
+    // first chunk's neighbour slots and couplings
+    Cursor nx{0u, 0u, first_slice(0)};
+    settle(nx);
+    uint4 nm = load_meta(nx);
+    Cursor nn = nx;  // the one after, of which only the meta data is read ahead
+    nn.slice += stride;
+    settle(nn);
+    uint4 nnm = load_meta(nn);
+    auto load_vi = [&](const Cursor& c) -> uint32_t {
+        return c.sweep < n_sweeps ? ld_stream_u32(d.vinfo + (int64_t)c.slice * 32 + lane, pol_stream) : kInactive;
+    };
+    uint32_t nvi = load_vi(nx), nnvi = load_vi(nn);
+    SpinWords<R> nsi;
+    uint32_t col[kChunk];
+    uint64_t J[kChunk];
+    int nkmin[R];
+#pragma unroll
+    for (int e = 0; e < kChunk; ++e) {
+        col[e] = 0u;
+        J[e] = 0ull;
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        nsi.v[r] = 0ull;
+        nkmin[r] = 0;
+    }
+    auto load_chunk = [&](uint32_t idx, uint32_t n) {
+#pragma unroll
+        for (int e = 0; e < kChunk; ++e) {
+            J[e] = 0ull;
+            if ((uint32_t)e < n) {
+                col[e] = ld_stream_u32(d.col + idx + 32 * e, pol_stream);
+                J[e] = ld_stream_u64(d.jb + idx + 32 * e, pol_stream);
+            }
+        }
+    };
+    auto load_slice = [&] {
+        if (nx.sweep < n_sweeps) {
+            const int64_t slot = (int64_t)nx.slice * 32 + lane;
+            nsi = ld_spins<R>(d.S + slot * R, pol_keep);
+            load_chunk(nm.x + lane, nm.y);
+        }
+    };
+    auto next_acceptance = [&] {
+        if (nx.sweep < n_sweeps)
+            accept_from<R>(nvi, t0 + nx.sweep, seeds[nm.z], thr + nm.z * (R * kVbThrStride), nkmin);
+    };
+    load_slice();
+
+    const uint32_t nq = n_sweeps * nc;
+    uint32_t sweep = 0, cls = 0, phase = 0;  // phases: spans between grid-wide barriers
+    bool ok = true;
+    for (uint32_t q = 0; q < nq; ++q) {
+        if (nx.sweep == sweep && nx.cls == cls) next_acceptance();
+        if (phase > 0 && cls <= tail && gridDim.x > 1) {
+            // admitted once every CTA has written the classes before (bounded; the polls are relaxed
+            // loads and one fence: an acquire in each would drop the L1 each time)
+            if (tid == 0) {
+                const uint32_t target = phase * gridDim.x;
+                int pass = ld_relaxed_u32(d.gbar) >= target;
+                if (!pass && d.stage_wait_ns) {
+                    const uint64_t ns0 = global_ns();
+                    for (uint32_t it = 1;; ++it) {
+                        if (ld_relaxed_u32(d.gbar) >= target) {
+                            pass = 1;
+                            break;
+                        }
+                        if ((it & 255u) == 0u && global_ns() - ns0 > d.stage_wait_ns) break;
+                    }
+                }
+                asm volatile("fence.acq_rel.gpu;" ::: "memory");
+                if (!pass) {
+                    atomicOr(d.err, 8);
+                    s_ok = 0;
+                }
+            }
+            __syncthreads();
+            ok = s_ok != 0;
+            if (!ok) break;  // uniform over the CTA
+        }
+        while (nx.sweep == sweep && nx.cls == cls) {
+            const uint32_t slice = nx.slice, vi = nvi;
+            SpinWords<R> si = nsi;
+            int kmin[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) kmin[r] = nkmin[r];
+            uint32_t left = nm.y, idx = nm.x + lane;
+            auto advance = [&] {
+                nx = nn;
+                nm = nnm;
+                nvi = nnvi;
+                nn.slice += stride;
+                settle(nn);
+                load_slice();
+                nnm = load_meta(nn);
+                nnvi = load_vi(nn);
+            };
+            if (left < (1u << kSweepPlanes)) {
+                uint64_t p[R][kSweepPlanes];
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+#pragma unroll
+                    for (int b = 0; b < kSweepPlanes; ++b) p[r][b] = 0ull;
+                for (;;) {
+                    SpinWords<R> g[kChunk];
+                    uint64_t Jc[kChunk];
+#pragma unroll
+                    for (int e = 0; e < kChunk; ++e) {
+                        g[e] = si;  // an absent entry counts nothing: x = 0
+                        Jc[e] = J[e];
+                        if ((uint32_t)e < left) g[e] = ld_spins<R>(d.S + (int64_t)col[e] * R, pol_keep);
+                    }
+                    const bool last = left <= (uint32_t)kChunk;
+                    if (!last) {
+                        left -= kChunk;
+                        idx += 32 * kChunk;
+                        load_chunk(idx, left);
+                    } else {
+                        advance();
+                    }
+#pragma unroll
+                    for (int r = 0; r < R; ++r) {
+                        uint64_t x[kChunk];
+#pragma unroll
+                        for (int e = 0; e < kChunk; ++e) x[e] = si.v[r] ^ g[e].v[r] ^ Jc[e];
+                        bitslice_add4<kSweepPlanes>(p[r], x[0], x[1], x[2], x[3]);
+                        if constexpr (kChunk == 8) bitslice_add4<kSweepPlanes>(p[r], x[4], x[5], x[6], x[7]);
+                    }
+                    if (last) break;
+                }
+#pragma unroll
+                for (int r = 0; r < R; ++r) si.v[r] ^= at_least<kSweepPlanes>(p[r], kmin[r]);
+            } else {
+                uint64_t p[R][6];
+#pragma unroll
+                for (int r = 0; r < R; ++r)
+#pragma unroll
+                    for (int b = 0; b < 6; ++b) p[r][b] = 0ull;
+                for (uint32_t e = 0; e < left; ++e, idx += 32) {
+                    const uint64_t Je = __ldg(d.jb + idx);
+                    const SpinWords<R> sj = ld_spins<R>(d.S + (int64_t)__ldg(d.col + idx) * R, pol_keep);
+#pragma unroll
+                    for (int r = 0; r < R; ++r) bitslice_add<6>(p[r], si.v[r] ^ sj.v[r] ^ Je);
+                }
+#pragma unroll
+                for (int r = 0; r < R; ++r) si.v[r] ^= at_least<6>(p[r], kmin[r]);
+                advance();
+            }
+            // a warp's only slice comes next again: its words were read ahead of this update
+            if (nx.slice == slice) nsi = si;
+            if (vi != kInactive)
+                store_words_keep<R>(d.S + ((int64_t)slice * 32 + lane) * R, si, pol_keep);
+            if (nx.sweep == sweep && nx.cls == cls) next_acceptance();
+        }
+        __syncthreads();  // this CTA's words of the class are written
+        if (tail <= cls && cls + 1 < nc) {  // the tail goes on
+            ++cls;
+            continue;
+        }
+        ++phase;
+        if (tid == 0 && gridDim.x > 1)
+            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(d.gbar) : "memory");
+        if (++cls == nc) {
+            cls = 0;
+            ++sweep;
+        }
+    }
+    // the last CTA to leave rearms the counters for the next launch (every CTA leaves, also after
+    // a wait that gave up, and none looks at the arrivals any more once it has counted itself out)
+    if (tid == 0) {
+        __threadfence();
+        if (atomicAdd(d.gbar + 1, 1u) == gridDim.x - 1) {
+            atomicExch(d.gbar, 0u);
+            atomicExch(d.gbar + 1, 0u);
+        }
+    }
+}
+
+template <int R, int CH>
+static int sweep_warps(int sms) { return SweepShape<R, CH>::threads / 32 * 2 * sms; }
+
+template <int R, int CH>
+static int launch_sweeps(const VbPackedDev& d, int max_class_slices, int sms, uint32_t t0,
+                         int n_sweeps, cudaStream_t st) {
+    constexpr int threads = SweepShape<R, CH>::threads, warps = threads / 32;
+    auto kern = k_vb_sweeps<R, CH>;
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, 0) != cudaSuccess ||
+        per_sm < 1)
+        return -1;
+    if (per_sm > 2) per_sm = 2;
+    // as many CTAs as the largest class fills; below one per SM four slices each (a barrier of few
+    // CTAs is no dearer, and their warps share the schedulers less)
+    int64_t grid = ((int64_t)max_class_slices + warps - 1) / warps;
+    if (grid < sms) grid = std::min<int64_t>(sms, ((int64_t)max_class_slices + 3) / 4);
+    grid = std::min<int64_t>(grid, (int64_t)sms * per_sm);
+    if (grid < 1 || max_class_slices <= warps) grid = 1;  // the first CTA does it all
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(threads);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, d, t0, (uint32_t)n_sweeps) == cudaSuccess ? 1 : -1;
+}
+
+// Chunks of 8 entries where every warp has at most one slice of a class: the class then takes as long
+// as its widest slice, and fewer rounds of gathers count for more than warps in flight (R = 2,
+// N = 65536: 15.6 us a sweep, 16.6 with chunks of 4; R = 4, N = 60000: 24.6, 27.1).  Beyond that the
+// registers are better spent on more warps (R = 2, bipartite N = 2^18: 10.3 us with chunks of 4,
+// 11.9 with 8; Poissonian N = 2^22: 128, 145; R = 4, N = 10^6: 80, 90).
+template <int R>
+static int launch_r(const VbPackedDev& d, int max_class_slices, uint32_t t0, int n_sweeps, cudaStream_t st) {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+        return -1;
+    if (max_class_slices <= sweep_warps<R, 8>(sms))
+        return launch_sweeps<R, 8>(d, max_class_slices, sms, t0, n_sweeps, st);
+    return launch_sweeps<R, 4>(d, max_class_slices, sms, t0, n_sweeps, st);
+}
+
+int vb_packed_sweeps(const VbPackedDev& d, int max_class_slices, uint32_t t0, int n_sweeps,
+                     cudaStream_t st) {
+    if (n_sweeps <= 0 || d.n_colours <= 0) return 0;
+    switch (d.R) {
+        case 1: return launch_r<1>(d, max_class_slices, t0, n_sweeps, st);
+        case 2: return launch_r<2>(d, max_class_slices, t0, n_sweeps, st);
+        case 4: return launch_r<4>(d, max_class_slices, t0, n_sweeps, st);
+        default: return -1;
+    }
+}
+
+}  // namespace sg
