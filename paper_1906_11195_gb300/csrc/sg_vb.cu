@@ -22,6 +22,7 @@
 #include "../../include/sg.h"
 #include "sg_internal.cuh"
 #include "sg_model.h"
+#include "vb_resident.h"
 
 namespace sg {
 namespace {
@@ -243,6 +244,7 @@ public:
             up((void*)pk_.slice_meta, h_slice_meta_.data(), h_slice_meta_.size() * sizeof(uint4));
             check_cuda(cudaMemsetAsync(pk_.err, 0, 4, st), "memset");
             check_cuda(cudaMemsetAsync(pk_.gbar, 0, 8, st), "memset");
+            up((void*)rs_.graph_class_slice, graph_class_slice_.data(), graph_class_slice_.size() * 4);
             up((void*)pk_.class_slice, colour_slice_.data(), colour_slice_.size() * 4);
             up((void*)pk_.jb, h_jb_.data(), h_jb_.size() * 8);
             std::vector<uint64_t> seeds(n_inst);
@@ -254,6 +256,7 @@ public:
             up((void*)pk_.up_slice_base, h_up_base_.data(), h_up_base_.size() * 4);
             launches += vb_packed_build_upper(pk_, st);  // from col and jb, on the device
             launches += vb_packed_init(pk_, st);
+            form_ = plan_resident() ? kResident : kGrid;
         } else {
             up((void*)pl_.row_ptr, h_row_ptr_.data(), h_row_ptr_.size() * 4);
             up((void*)pl_.col, h_col_i_.data(), h_col_i_.size() * 4);
@@ -273,6 +276,63 @@ public:
         check_cuda(cudaStreamSynchronize(st), "attach");
     }
 
+    // The plan with 2^lc CTAs for every graph; false: some graph does not fit.
+    bool resident_layout(uint32_t lc, VbResident& rs) const {
+        const int nc = pk_.n_colours;
+        const uint32_t C = 1u << lc;
+        rs = rs_;
+        rs.cluster = C;
+        rs.log_cluster = lc;
+        rs.max_slices = 0;
+        rs.max_entries = 0;
+        for (int b = 0; b < n_inst; ++b) {
+            int64_t ns[kResMaxCluster] = {}, ne[kResMaxCluster] = {};
+            for (int c = 0; c < nc; ++c) {
+                const uint32_t lo = graph_class_slice_[(size_t)c * n_inst + b],
+                               hi = graph_class_slice_[(size_t)c * n_inst + b + 1];
+                if (hi - lo > C * 1024u) return false;  // far beyond shared memory
+                for (uint32_t s = lo; s < hi; ++s) {
+                    const uint32_t k = (s - lo) & (C - 1);
+                    ++ns[k];
+                    ne[k] += h_slice_base_[s + 1] - h_slice_base_[s];
+                }
+            }
+            for (uint32_t k = 0; k < C; ++k) {
+                rs.max_slices = std::max(rs.max_slices, (int)ns[k]);
+                rs.max_entries = std::max(rs.max_entries, (uint32_t)ne[k]);
+            }
+            if (vb_resident_smem(R, rs.max_slices, rs.max_entries) > (size_t)kResMaxSmem) return false;
+        }
+        return vb_resident_clusters(R, rs) >= n_inst;
+    }
+
+    // Which graphs run in shared memory, and on how many CTAs each (R = 2, degree 4, us a sweep).  One
+    // CTA as long as its 12 updating warps take a class in two rounds at most: N = 1000 4.8, against
+    // 6.1 in a cluster and 11.4 in the grid-wide form; N = 2500 8.3 against 6.6 in a cluster of 16.
+    // Otherwise the largest cluster that the GPU holds for every graph of the batch (N = 8000: 14.5
+    // with 4 CTAs, 10.7 with 8, 8.5 with 16; grid-wide 15.1), up to 104 KB of words gathered by a CTA in a
+    // sweep: gathers from other CTAs' shared memory take about 4 cycles for each 16 bytes, and there
+    // the grid-wide form draws level (N = 40000, 170 KB: 22.9 against 16.9; N = 20011 with four
+    // replicas, 175 KB: 22.7 against 18.3).
+    bool plan_resident() {
+        constexpr int64_t kMaxGatherBytes = 104 * 1024;
+        if (pk_.n_colours < 1) return false;
+        int widest = 0;  // slices of the largest class of one graph
+        for (size_t i = 0; i + 1 < graph_class_slice_.size(); ++i)
+            widest = std::max(widest, (int)(graph_class_slice_[i + 1] - graph_class_slice_[i]));
+        VbResident rs;
+        if (widest <= kResMain + kResMain / 3 && resident_layout(0, rs)) {
+            rs_ = rs;
+            return true;
+        }
+        for (uint32_t lc = 4; lc >= 1; --lc)
+            if (resident_layout(lc, rs) && (int64_t)rs.max_entries * R * 8 <= kMaxGatherBytes) {
+                rs_ = rs;
+                return true;
+            }
+        return false;
+    }
+
     // The packed sweeps of a call, without a captured graph: a launch takes as many sweeps as run in a few
     // milliseconds, so nothing is left of the launches' gaps.
     bool sweep_direct(int64_t t0, int64_t n, cudaStream_t st) override {
@@ -281,7 +341,8 @@ public:
         for (int64_t done = 0; done < n;) {
             const int m = (int)std::min<int64_t>(n - done, most);
             const uint32_t t = (uint32_t)(t0 + done);
-            const int k = vb_packed_sweeps(pk_, max_class_slices_, t, m, st);
+            const int k = form_ == kResident ? vb_resident_sweeps(pk_, rs_, t, m, st)
+                                             : vb_packed_sweeps(pk_, max_class_slices_, t, m, st);
             if (k < 0) fail(SG_ECUDA, "sweep launch failed");
             launches += k;
             done += m;
@@ -542,6 +603,7 @@ private:
             pk_.slice_meta = c.take<uint4>(h_slice_meta_.size());
             pk_.err = c.take<int>(1);
             pk_.gbar = c.take<uint32_t>(2);
+            rs_.graph_class_slice = c.take<uint32_t>(graph_class_slice_.size());
             pk_.class_slice = c.take<uint32_t>(colour_slice_.size());
             // about 96 MB of the 129 MB L2 for graph and spins together
             pk_.stream_first = h_col_.size() * 12 + (size_t)n_slots_ * (4 + 8 * R) > ((size_t)96 << 20);
@@ -648,6 +710,7 @@ private:
             colour_slice_[c] = (uint32_t)(cursor / 32);
             for (int b = 0; b < n_inst; ++b) {
                 const Graph& g = graphs_[b];
+                graph_class_slice_.push_back((uint32_t)(cursor / 32));
                 if (c >= g.n_colours) continue;
                 const int64_t start = cursor;
                 // highest degree first: the longest slices start early instead of forming the tail
@@ -666,6 +729,7 @@ private:
             }
         }
         colour_slice_[cmax] = (uint32_t)(cursor / 32);
+        graph_class_slice_.push_back((uint32_t)(cursor / 32));
         for (int c = 0; c < cmax; ++c)
             max_class_slices_ = std::max(max_class_slices_, (int)(colour_slice_[c + 1] - colour_slice_[c]));
         n_slots_ = cursor;
@@ -761,7 +825,11 @@ private:
     }
 
     int kernel_ = SG_VB_PACKED;
+    enum Form { kGrid, kResident };
+    Form form_ = kGrid;         // vb_sweep.cu or vb_resident.cu, chosen at attach
     int max_class_slices_ = 0;  // slices of the largest class
+    VbResident rs_{};
+    std::vector<uint32_t> graph_class_slice_;  // first slice of every (class, graph)
     int Lc_ = 64;
     size_t ws_bytes_ = 0;
     std::vector<Graph> graphs_;
