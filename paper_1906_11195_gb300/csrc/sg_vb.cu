@@ -277,20 +277,23 @@ public:
     }
 
     // The plan with 2^lc CTAs for every graph; false: some graph does not fit.
-    bool resident_layout(uint32_t lc, VbResident& rs) const {
+    bool resident_layout(uint32_t lc, bool copies, VbResident& rs) const {
         const int nc = pk_.n_colours;
         const uint32_t C = 1u << lc;
         rs = rs_;
         rs.cluster = C;
         rs.log_cluster = lc;
+        rs.copies = copies;
+        rs.graph_slices = 0;
         rs.max_slices = 0;
         rs.max_entries = 0;
         for (int b = 0; b < n_inst; ++b) {
-            int64_t ns[kResMaxCluster] = {}, ne[kResMaxCluster] = {};
+            int64_t ns[kResMaxCluster] = {}, ne[kResMaxCluster] = {}, all = 0;
             for (int c = 0; c < nc; ++c) {
                 const uint32_t lo = graph_class_slice_[(size_t)c * n_inst + b],
                                hi = graph_class_slice_[(size_t)c * n_inst + b + 1];
                 if (hi - lo > C * 1024u) return false;  // far beyond shared memory
+                all += hi - lo;
                 for (uint32_t s = lo; s < hi; ++s) {
                     const uint32_t k = (s - lo) & (C - 1);
                     ++ns[k];
@@ -301,36 +304,46 @@ public:
                 rs.max_slices = std::max(rs.max_slices, (int)ns[k]);
                 rs.max_entries = std::max(rs.max_entries, (uint32_t)ne[k]);
             }
-            if (vb_resident_smem(R, rs.max_slices, rs.max_entries) > (size_t)kResMaxSmem) return false;
+            rs.graph_slices = std::max(rs.graph_slices, (int)all);
+            if (vb_resident_smem(R, copies ? rs.graph_slices : rs.max_slices, rs.max_slices,
+                                 rs.max_entries) > (size_t)kResMaxSmem)
+                return false;
         }
         return vb_resident_clusters(R, rs) >= n_inst;
     }
 
-    // Which graphs run in shared memory, and on how many CTAs each (R = 2, degree 4, us a sweep).  One
-    // CTA as long as its 12 updating warps take a class in two rounds at most: N = 1000 4.8, against
-    // 6.1 in a cluster and 11.4 in the grid-wide form; N = 2500 8.3 against 6.6 in a cluster of 16.
-    // Otherwise the largest cluster that the GPU holds for every graph of the batch (N = 8000: 14.5
-    // with 4 CTAs, 10.7 with 8, 8.5 with 16; grid-wide 15.1), up to 104 KB of words gathered by a CTA in a
-    // sweep: gathers from other CTAs' shared memory take about 4 cycles for each 16 bytes, and there
-    // the grid-wide form draws level (N = 40000, 170 KB: 22.9 against 16.9; N = 20011 with four
-    // replicas, 175 KB: 22.7 against 18.3).
+    // Which graphs run in shared memory, and how (R = 2, Poissonian of degree 4, us a sweep).
+    // One CTA as long as its 12 updating warps take a class in two rounds at most: N = 1000 4.5,
+    // against 4.8 in a cluster and 11.4 in the grid-wide form; N = 2500 7.8, 5.0 in a cluster.
+    // A cluster whose CTAs each hold a copy of all words: 8 CTAs where that fits (N = 2500 5.0, 16 CTAs
+    // 5.5, without copies 6.3; N = 6000 6.4, 6.9, 7.6), else 16 (N = 9000 8.1, without copies 8.6;
+    // one replica, N = 18000 8.3, 11.4).  Each update goes to all CTAs, so four replicas do not gain
+    // from 16 (N = 4500 13.6, without copies 10.9), nor does a graph of degree 4, whose words
+    // arrive in one round (bipartite N = 4096: 16 CTAs without copies 2.9, 8 with copies 3.2).
+    // Without copies up to 104 KB of words gathered by a CTA in a sweep: gathers from other CTAs' shared
+    // memory take about 4 cycles for each 16 bytes, and there the grid-wide form draws level
+    // (N = 40000, 170 KB: 22.9 against 16.9; N = 20011, four replicas, 175 KB: 22.7 against 18.3).
+    // A batch takes the first of these for which the GPU holds all its clusters at once.
     bool plan_resident() {
         constexpr int64_t kMaxGatherBytes = 104 * 1024;
         if (pk_.n_colours < 1) return false;
         int widest = 0;  // slices of the largest class of one graph
         for (size_t i = 0; i + 1 < graph_class_slice_.size(); ++i)
             widest = std::max(widest, (int)(graph_class_slice_[i + 1] - graph_class_slice_[i]));
+        uint32_t width = 0;  // entries of the widest slice
+        for (size_t i = 0; i + 1 < h_slice_base_.size(); ++i)
+            width = std::max(width, (h_slice_base_[i + 1] - h_slice_base_[i]) / 32);
         VbResident rs;
-        if (widest <= kResMain + kResMain / 3 && resident_layout(0, rs)) {
+        auto take = [&](uint32_t lc, bool copies) {
+            if (!resident_layout(lc, copies, rs)) return false;
+            if (lc > 0 && !copies && (int64_t)rs.max_entries * R * 8 > kMaxGatherBytes) return false;
             rs_ = rs;
             return true;
-        }
-        for (uint32_t lc = 4; lc >= 1; --lc)
-            if (resident_layout(lc, rs) && (int64_t)rs.max_entries * R * 8 <= kMaxGatherBytes) {
-                rs_ = rs;
-                return true;
-            }
-        return false;
+        };
+        if (widest <= kResMain + kResMain / 3 && take(0, false)) return true;
+        if (width <= 4 && R >= 2 && take(4, false)) return true;
+        return take(3, true) || (R < 4 && take(4, true)) || take(4, false) || take(2, true) ||
+               take(3, false) || take(1, true) || take(2, false) || take(1, false);
     }
 
     // The packed sweeps of a call, without a captured graph: a launch takes as many sweeps as run in a few

@@ -10,8 +10,13 @@
 // (a CTA barrier for one CTA) instead of a grid-wide one through L2.  Six of
 // the 18 warps work out the acceptance of a class for the next sweep while the others update it.
 //
-// us a sweep, before (grid-wide: vb_sweep.cu's predecessor) -> now: N = 1000 18 -> 4.8 (one CTA),
-// bipartite N = 4096 9.8 -> 3.0, N = 8000 15 (vb_sweep.cu) -> 8.4 (clusters of 16).
+// In a cluster the words that neighbours read are either where their owner keeps them, or every
+// CTA holds a copy of all words: gathers from another CTA take about 4 cycles for each 16 bytes, so
+// where the copies fit it is cheaper to send every updated slice to the other CTAs (512 bytes for two
+// replicas, whole lines, about 43 cycles each) and gather at home.
+//
+// us a sweep, two replicas, before (grid-wide) -> now: N = 1000 18 -> 4.5 (one CTA), 2500 12.4 -> 5.0,
+// bipartite 4096 9.8 -> 2.9, 6000 14 -> 6.4, 9000 15 -> 8.1.
 //
 // The slices (32 vertices) of a class are dealt in turn to the CTAs of the cluster, and in a CTA to
 // its warps.
@@ -41,18 +46,29 @@ template <int R, int MODE>
 __device__ __forceinline__ SpinWords<R> gather_near(uint32_t a) {
     SpinWords<R> s;
     if constexpr (R == 1) {
-        if constexpr (MODE == kResSolo) asm volatile("ld.shared.u64 %0, [%1];" : "=l"(s.v[0]) : "r"(a));
+        if constexpr (MODE != kResCluster) asm volatile("ld.shared.u64 %0, [%1];" : "=l"(s.v[0]) : "r"(a));
         else asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(s.v[0]) : "r"(a));
     } else {
 #pragma unroll
         for (int h = 0; h < R / 2; ++h) {
-            if constexpr (MODE == kResSolo)
+            if constexpr (MODE != kResCluster)
                 asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(s.v[2 * h]), "=l"(s.v[2 * h + 1]) : "r"(a + 16 * h));
             else
                 asm volatile("ld.shared::cluster.v2.u64 {%0, %1}, [%2];" : "=l"(s.v[2 * h]), "=l"(s.v[2 * h + 1]) : "r"(a + 16 * h));
         }
     }
     return s;
+}
+
+template <int R>
+__device__ __forceinline__ void store_remote(uint32_t a, const SpinWords<R>& s) {
+    if constexpr (R == 1) {
+        asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(a), "l"(s.v[0]) : "memory");
+    } else {
+#pragma unroll
+        for (int h = 0; h < R / 2; ++h)
+            asm volatile("st.shared::cluster.v2.u64 [%0], {%1, %2};" ::"r"(a + 16 * h), "l"(s.v[2 * h]), "l"(s.v[2 * h + 1]) : "memory");
+    }
 }
 
 // every thread's words of a class are visible to the cluster, and no thread reads on before
@@ -74,9 +90,10 @@ __global__ void __launch_bounds__(kResThreads, 1)
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ uint32_t c_lo[kVbMaxColours], c_hi[kVbMaxColours];       // slices of the graph's classes
     __shared__ uint16_t first_of[kVbMaxColours + 1][kResMaxCluster];    // local slices before a class, per CTA
+    __shared__ uint32_t c_before[kVbMaxColours + 1];                    // the graph's slices before a class
     __shared__ __align__(16) uint32_t thr[R * kVbThrStride];
     uint64_t* S = reinterpret_cast<uint64_t*>(smem);                            // [slots][R]
-    uint64_t* J = S + (size_t)rs.max_slices * 32 * R;                           // [entries]
+    uint64_t* J = S + (size_t)(MODE == kResCopies ? rs.graph_slices : rs.max_slices) * 32 * R;                           // [entries]
     uint32_t* nbr = reinterpret_cast<uint32_t*>(J + rs.max_entries);            // [entries] address of the words
     uint32_t* vinfo = nbr + rs.max_entries;                                     // [slots]
     uint32_t* base = vinfo + rs.max_slices * 32;                                // [slices + 1] first entry
@@ -96,6 +113,13 @@ __global__ void __launch_bounds__(kResThreads, 1)
     for (uint32_t i = tid; i < (uint32_t)(R * kVbThrStride); i += kResThreads)
         thr[i] = __ldg(d.thr + g * (R * kVbThrStride) + i);
     __syncthreads();
+    if (tid == 0) {
+        uint32_t n = 0;
+        for (uint32_t c = 0; c < nc; ++c) {
+            c_before[c] = n;
+            n += c_hi[c] - c_lo[c];
+        }
+    }
     if (tid < C) {
         uint32_t n = 0;
         for (uint32_t c = 0; c < nc; ++c) {
@@ -139,9 +163,11 @@ __global__ void __launch_bounds__(kResThreads, 1)
         const uint32_t s = slice_of(l);
         const uint32_t slot = s * 32 + lane;
         vinfo[l * 32 + lane] = __ldg(d.vinfo + slot);
-        const SpinWords<R> w = load_words<R>(d.S + (int64_t)slot * R);
+        if constexpr (MODE != kResCopies) {
+            const SpinWords<R> w = load_words<R>(d.S + (int64_t)slot * R);
 #pragma unroll
-        for (int r = 0; r < R; ++r) S[(l * 32 + lane) * R + r] = w.v[r];
+            for (int r = 0; r < R; ++r) S[(l * 32 + lane) * R + r] = w.v[r];
+        }
         const uint32_t gb = __ldg(d.slice_base + s);
         for (uint32_t e = base[l] + lane; e < base[l + 1]; e += 32) {
             const uint32_t ge = gb + (e - base[l]);
@@ -149,10 +175,22 @@ __global__ void __launch_bounds__(kResThreads, 1)
             const uint32_t j = __ldg(d.col + ge), sj = j >> 5;
             uint32_t c = 0;
             while (sj < c_lo[c] || sj >= c_hi[c]) ++c;  // every neighbour lies in a class of this graph
+            if constexpr (MODE == kResCopies) {
+                nbr[e] = smem_addr(S + ((c_before[c] + sj - c_lo[c]) * 32 + (j & 31u)) * R);
+                continue;
+            }
             const uint32_t i = sj - c_lo[c], owner = i & (C - 1u);
             const uint32_t a = smem_addr(S + ((first_of[c][owner] + (i >> lc)) * 32 + (j & 31u)) * R);
             nbr[e] = MODE == kResSolo ? a : cluster_addr(a, owner);
         }
+    }
+    if constexpr (MODE == kResCopies) {  // all the graph's words
+        for (uint32_t c = 0; c < nc; ++c)
+            for (uint32_t i = tid; i < (c_hi[c] - c_lo[c]) * 32; i += kResThreads) {
+                const SpinWords<R> w = load_words<R>(d.S + ((int64_t)c_lo[c] * 32 + i) * R);
+#pragma unroll
+                for (int r = 0; r < R; ++r) S[((size_t)c_before[c] * 32 + i) * R + r] = w.v[r];
+            }
     }
     // Acceptance of the vertices of local slice l at time t: a lane flips iff its unsatisfied count u
     // reaches ceil((d - m*) / 2), m* the largest accepted m (the accepted m are a prefix 1..m*)
@@ -192,7 +230,8 @@ __global__ void __launch_bounds__(kResThreads, 1)
                     accept(l, t + 1);
             }
             for (uint32_t l = warp < kResMain ? first_of[c][rank] + warp : l_end; l < l_end; l += kResMain) {
-                uint64_t* own = S + (l * 32 + lane) * R;
+                const uint32_t i = ((l - first_of[c][rank]) << lc) + rank;  // the slice's place in its class
+                uint64_t* own = S + ((MODE == kResCopies ? c_before[c] + i : l) * 32 + lane) * R;
                 SpinWords<R> si = load_words<R>(own);
                 uint32_t e = base[l] + lane;
                 const uint32_t end = base[l + 1];  // width = (end - base[l]) / 32
@@ -255,20 +294,30 @@ __global__ void __launch_bounds__(kResThreads, 1)
                 if (vi != kInactive) {
 #pragma unroll
                     for (int r = 0; r < R; ++r) own[r] = si.v[r];
+                    if constexpr (MODE == kResCopies) {
+                        const uint32_t a = smem_addr(own);
+                        for (uint32_t k = 1; k < C; ++k) store_remote<R>(cluster_addr(a, (rank + k) & (C - 1u)), si);
+                    }
                 }
             }
             class_barrier_arrive<MODE>();
         }
     class_barrier_wait<MODE>();  // no CTA leaves while another may read its words
     for (uint32_t l = warp; l < n_local; l += warps) {
-        const uint32_t slot = slice_of(l) * 32 + lane;
+        const uint32_t s = slice_of(l);
+        uint32_t at = l;
+        if constexpr (MODE == kResCopies) {
+            uint32_t c = 0;
+            while (l >= first_of[c + 1][rank]) ++c;
+            at = c_before[c] + s - c_lo[c];
+        }
 #pragma unroll
-        for (int r = 0; r < R; ++r) d.S[(int64_t)slot * R + r] = S[(l * 32 + lane) * R + r];
+        for (int r = 0; r < R; ++r) d.S[((int64_t)s * 32 + lane) * R + r] = S[(at * 32 + lane) * R + r];
     }
 }
 
-size_t vb_resident_smem(int R, int max_slices, int64_t max_entries) {
-    return (size_t)max_slices * 32 * R * 8 + (size_t)max_entries * 12 + (size_t)max_slices * 32 * 4 +
+size_t vb_resident_smem(int R, int word_slices, int max_slices, int64_t max_entries) {
+    return (size_t)word_slices * 32 * R * 8 + (size_t)max_entries * 12 + (size_t)max_slices * 32 * 4 +
            ((size_t)max_slices + 1) * 4 + (size_t)max_slices * 64 * R;
 }
 
@@ -276,7 +325,7 @@ template <int R, int MODE>
 static cudaError_t resident_config(const VbResident& rs, int n_graphs, cudaLaunchConfig_t& cfg,
                                    cudaLaunchAttribute* attr) {
     auto kern = k_vb_resident<R, MODE>;
-    const size_t smem = vb_resident_smem(R, rs.max_slices, rs.max_entries);
+    const size_t smem = vb_resident_smem(R, rs.copies ? rs.graph_slices : rs.max_slices, rs.max_slices, rs.max_entries);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kResMaxSmem);
     if (e != cudaSuccess) return e;
     if (MODE != kResSolo) {
@@ -326,11 +375,12 @@ static int resident_clusters(const VbResident& rs) {
 template <int R>
 static int resident_clusters_mode(const VbResident& rs) {
     return rs.cluster == 1 ? resident_clusters<R, kResSolo>(rs)
+           : rs.copies ? resident_clusters<R, kResCopies>(rs)
                                : resident_clusters<R, kResCluster>(rs);
 }
 
 int vb_resident_clusters(int R, const VbResident& rs) {
-    if (vb_resident_smem(R, rs.max_slices, rs.max_entries) > (size_t)kResMaxSmem) return 0;
+    if (vb_resident_smem(R, rs.copies ? rs.graph_slices : rs.max_slices, rs.max_slices, rs.max_entries) > (size_t)kResMaxSmem) return 0;
     switch (R) {
         case 1: return resident_clusters_mode<1>(rs);
         case 2: return resident_clusters_mode<2>(rs);
@@ -354,6 +404,7 @@ template <int R>
 static int resident_launch_mode(const VbPackedDev& d, const VbResident& rs, uint32_t t0,
                                 int n_sweeps, cudaStream_t st) {
     return rs.cluster == 1 ? resident_launch<R, kResSolo>(d, rs, t0, n_sweeps, st)
+           : rs.copies ? resident_launch<R, kResCopies>(d, rs, t0, n_sweeps, st)
                                : resident_launch<R, kResCluster>(d, rs, t0, n_sweeps, st);
 }
 
