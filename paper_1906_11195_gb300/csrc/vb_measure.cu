@@ -127,8 +127,12 @@ __device__ __forceinline__ void count_rows(const VbPackedDev& d, const uint64_t*
     }
 }
 
+// CTAs that share an SM (64 registers a thread for one and two replicas, 128 for four)
 template <int R>
-__global__ void __launch_bounds__(32 * kMeasureWarps)
+constexpr int kMeasureCtas = R == 4 ? 2 : 4;
+
+template <int R>
+__global__ void __launch_bounds__(32 * kMeasureWarps, kMeasureCtas<R>)
     k_vb_packed_measure(VbPackedDev d, VbMeasure m, MeasureGrid mg) {
     __shared__ unsigned long long acc[R * 64];
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
@@ -218,9 +222,15 @@ int vb_packed_measure(const VbPackedDev& d, const VbMeasure& m, cudaStream_t st)
     if (rows == 0) return 0;
     MeasureGrid mg;
     mg.up_rows = d.up_rows;
-    // about 32 warps for each of the 152 SMs
-    int64_t run = (rows + 152 * 32 - 1) / (152 * 32);
-    if (run > kMeasureRun) run = kMeasureRun;
+    // whole waves of the CTAs that the 152 SMs hold at once, a run as long as that allows
+    const int64_t slots = 152 * (d.R == 4 ? kMeasureCtas<4> : kMeasureCtas<2>);
+    const int64_t waves = (rows + slots * kMeasureWarps * kMeasureRun - 1) / (slots * kMeasureWarps * kMeasureRun);
+    int64_t run = (rows + waves * slots * kMeasureWarps - 1) / (waves * slots * kMeasureWarps);
+    auto ctas = [&](int64_t r) {  // each pass's last CTA is part empty
+        const int64_t n = r * kMeasureWarps;
+        return (d.n_slices + n - 1) / n * passes + (m.e ? ((int64_t)d.up_rows + n - 1) / n : 0);
+    };
+    while (run < kMeasureRun && ctas(run) > waves * slots) ++run;
     mg.run_s = mg.run_e = (int)run;
     const int64_t per_cta = run * kMeasureWarps;
     mg.nb_s = passes ? (uint32_t)((d.n_slices + per_cta - 1) / per_cta) : 1u;
