@@ -17,17 +17,24 @@
 //     H_ready of that tile is raised to k + L + 2.
 //
 //   chain CTAs (the next nC): CTA c owns replicas W c .. W c + W - 1, one warp per replica, plus
-//     a staging warp.  For block k the staging warp loads (TMA, into a ring of shared-memory
-//     stages) the couplings of block b's rows with the columns of blocks k - L .. k (as bits),
-//     the replicas' K* (the largest accepted k of each spin's random number, computed for all
-//     sweeps of the launch before it starts) and the fields of block b's rows: from H itself
-//     for k <= L (nothing of
-//     this launch has reached them through the tensor cores yet), else from Hpub once H_ready
-//     says it holds every block before k - L.  The replica warp adds the flips of blocks
-//     k - L .. k - 1 of this launch (its own, kept in shared memory) with popcounts over the
-//     coupling bits, then takes the 128 sequential decisions (ballot per accepted flip, as in
-//     the in-block kernel) and writes 2 D_k into ring slot k mod Q.  The staging warp raises
+//     a fold warp for each, a staging, a fields and a release warp.  For block k the staging warp
+//     loads (TMA, into a ring of shared-memory stages) the couplings of block b's rows with the
+//     columns of blocks k - L .. k (as bits) and the replicas' K* (the largest accepted k of each
+//     spin's random number, computed for all sweeps of the launch before it starts); the fields
+//     warp loads the fields of block b's rows: from H itself for k <= L (nothing of this launch
+//     has reached them through the tensor cores yet), else from Hpub once H_ready says it holds
+//     every block before k - L.  The fold and replica warps add the flips of blocks
+//     k - L .. k - 1 of this launch (its own, kept in shared memory) with counts over the coupling
+//     bits; the replica warp then takes the 128 sequential decisions (ballot per accepted flip, as in
+//     the in-block kernel) and writes 2 D_k into ring slot k mod Q.  The release warp raises
 //     D_count[slot] once every replica warp of the CTA is done with the block.
+//
+// What bounds it: latency, of the decisions and of the way round from a block's decisions to the fields
+// that hold them.  Nothing that can be done earlier sits on that way: the couplings are staged apart from
+// the fields, and the fold of blocks k - L .. k - 3 is done before the fields arrive.  us a sweep
+// (64-sweep launches), fields staged with the couplings -> apart: N = 8192, R = 256 102.3 -> 95.1,
+// N = 4096, R = 128 46.5 -> 42.3.  Measured and left: L = 4 122.6, L = 8 94.3 (N = 4096 45.0, 42.3 with
+// L = 6); the spin changes written by the release warp instead of the replica warps 96.2.
 //
 // So the sequential chain of a replica never waits for a launch or for the tensor cores, as
 // long as the field CTAs publish a tile within L chain blocks; it needs L < nb so that a fold
@@ -396,11 +403,12 @@ __device__ void persist_field_cta(const CUtensorMap* mapJ, const CUtensorMap* ma
 
 // ------------------------------------------------------------------------------------------
 // chain CTA: warps 0..W-1 are the replicas' chains, warps W..2W-1 their fold warps, warp 2W
-// (lane 0) stages the blocks, warp 2W + 1 (lane 0) tells the field CTAs (D_count) when every
-// replica warp has written a block's spin changes.  For block k the fold warp of replica w adds to the staged fields
-// the flips of blocks k - L .. k - 2 (complete while the chain runs block k - 1) and hands the
-// result over in shared memory; the chain warp adds block k - 1's flips itself (16 popcounts
-// per lane) and takes the decisions.  So only one block's fold sits on the chain.
+// (lane 0) stages the blocks' couplings, warp 2W + 2 (lane 0) their fields, warp 2W + 1 (lane 0)
+// tells the field CTAs (D_count) when every replica warp has written a block's spin changes.  For
+// block k the fold warp of replica w counts the flips of blocks k - L .. k - 3, then of k - 2 (complete
+// while the chain runs block k - 1), adds them to the fields once these are staged and hands the
+// result over in shared memory; the chain warp adds block k - 1's flips itself (16 popcounts per
+// lane) and takes the decisions.  So only one block's fold sits on the chain.
 // ------------------------------------------------------------------------------------------
 __device__ __forceinline__ void fold_block(int (&h)[4], const uint32_t* Jp, const uint32_t* Fw,
                                            const uint32_t* Sw, int bp, bool live, uint32_t lane) {
@@ -417,6 +425,70 @@ __device__ __forceinline__ void fold_block(int (&h)[4], const uint32_t* Jp, cons
         const int pf = __popc(Fv[cp]);
 #pragma unroll
         for (int q = 0; q < 4; ++q) h[q] += 2 * (pf - 2 * __popc(Fv[cp] & (jv[cp][q] ^ sv[cp])));
+    }
+}
+
+// The same for NB consecutive blocks, the first at bp0 (negative: cyclic in the nb blocks; k0 < 0: the
+// launch has no such block yet), into fresh h.  A population count issues at an eighth of the rate of a
+// logic operation, so eight words at a time go through carry-save adders into five counters, of which
+// the population is taken at the end; the flips are counted once, a word per lane.
+template <int NB>
+__device__ __forceinline__ void fold_window(int (&h)[4], const uint32_t* Jw, const uint32_t* Fw,
+                                            const uint32_t* Sw, int bp0, int nb, int k0, uint32_t lane) {
+    static_assert(NB % 2 == 0 && NB <= 6, "eight words at a time, at most 24 counted");
+    uint32_t mine = 0u;
+    {
+        const int i = (int)(lane >> 2), bp = bp0 + i;
+        if (i < NB && k0 + i >= 0) mine = Fw[(bp < 0 ? bp + nb : bp) * 4 + (lane & 3)];
+    }
+    const int flips = __reduce_add_sync(0xFFFFFFFFu, (unsigned)__popc(mine));
+    uint32_t p[4][5];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int c = 0; c < 5; ++c) p[q][c] = 0u;
+    auto add = [](uint32_t& s, uint32_t a, uint32_t b) -> uint32_t {  // s += a + b, carry out
+        const uint32_t t = s, x = t ^ a;
+        s = x ^ b;
+        return (t & a) | (b & x);
+    };
+#pragma unroll
+    for (int i = 0; i < NB; i += 2) {
+        uint32_t F[8], S[8];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            int bp = bp0 + i + u;
+            if (bp < 0) bp += nb;
+            const uint4 f = *reinterpret_cast<const uint4*>(Fw + bp * 4), sv = *reinterpret_cast<const uint4*>(Sw + bp * 4);
+            const bool live = k0 + i + u >= 0;
+            F[4 * u] = live ? f.x : 0u;
+            F[4 * u + 1] = live ? f.y : 0u;
+            F[4 * u + 2] = live ? f.z : 0u;
+            F[4 * u + 3] = live ? f.w : 0u;
+            S[4 * u] = sv.x;
+            S[4 * u + 1] = sv.y;
+            S[4 * u + 2] = sv.z;
+            S[4 * u + 3] = sv.w;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            uint32_t x[8];
+#pragma unroll
+            for (int w = 0; w < 8; ++w) x[w] = F[w] & (Jw[(i * 4 + w) * 128 + 32 * q + lane] ^ S[w]);
+            const uint32_t c0 = add(p[q][0], x[0], x[1]), c1 = add(p[q][0], x[2], x[3]);
+            const uint32_t c2 = add(p[q][0], x[4], x[5]), c3 = add(p[q][0], x[6], x[7]);
+            const uint32_t d0 = add(p[q][1], c0, c1), d1 = add(p[q][1], c2, c3);
+            const uint32_t e0 = add(p[q][2], d0, d1);
+            const uint32_t f0 = p[q][3] & e0;
+            p[q][3] ^= e0;
+            p[q][4] ^= f0;  // 24 < 32: no carry
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int n = __popc(p[q][0]) + 2 * __popc(p[q][1]) + 4 * __popc(p[q][2]) + 8 * __popc(p[q][3]) +
+                      16 * __popc(p[q][4]);
+        h[q] = 2 * (flips - 2 * n);
     }
 }
 
@@ -441,6 +513,7 @@ __device__ void persist_chain_cta(const SkDev& d, const SkPersistArgs& a, const 
     uint64_t* emptyc = bars + kChainStages;   // [kChainStages]: chain and fold warps done
     uint64_t* cdone = bars + 2 * kChainStages;    // [W][2]: the chain finished block k (k & 1)
     uint64_t* hrdy = cdone + 2 * W;               // [W][2]: folded fields of block k (k & 1)
+    uint64_t* fullh = hrdy + 2 * W;               // [kChainStages]: the stage's fields landed
     uint32_t* D_count = a.sync;
     uint32_t* D_free = a.sync + Q;
     uint32_t* H_ready = a.sync + 2 * Q;
@@ -449,6 +522,7 @@ __device__ void persist_chain_cta(const SkDev& d, const SkPersistArgs& a, const 
         for (int s = 0; s < kChainStages; ++s) {
             mbar_init(&fullc[s], 1);
             mbar_init(&emptyc[s], 2 * W);
+            mbar_init(&fullh[s], 1);
         }
         for (int i = 0; i < 4 * W; ++i) mbar_init(&cdone[i], 1);  // cdone and hrdy
         for (int w = 0; w < W; ++w) done_cnt[w] = 0u;
@@ -464,12 +538,11 @@ __device__ void persist_chain_cta(const SkDev& d, const SkPersistArgs& a, const 
     __syncthreads();
 
     if (warp == 2 * W) {
-        // ---------------- staging warp: block k (couplings, K*, fields) ----------------
+        // ---------------- staging warp: couplings and K* of block k ----------------
         if (lane == 0) {
-            const uint32_t stage_tx = (uint32_t)chain_stage_bytes(W, L);
+            const uint32_t stage_tx = (uint32_t)(chain_stage_bytes(W, L) - (size_t)W * 128 * 4);
             const uint64_t pol = l2_evict_last();
             asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&m.jb)) : "memory");
-            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&m.hpub)) : "memory");
             int last_fill[kChainStages];
             for (int s = 0; s < kChainStages; ++s) last_fill[s] = -1;
             auto prefetch = [&](int k) -> bool {
@@ -480,16 +553,9 @@ __device__ void persist_chain_cta(const SkDev& d, const SkPersistArgs& a, const 
                     atomicOr(d.err, 512);
                     return false;
                 }
-                const bool pub = k > L;
-                if (pub && !wait_at_least(&H_ready[b], (uint32_t)(k + 1), d.err, nowait)) {
-                    atomicOr(d.err, 1024);
-                    return false;
-                }
-                if (pub) fence_proxy_async_global();  // the fields were written by generic stores
                 uint8_t* st = ring + (size_t)s * stb;
                 uint32_t* Jw = reinterpret_cast<uint32_t*>(st);                    // [(L+1)*4][128]
                 int16_t* ks = reinterpret_cast<int16_t*>(Jw + (L + 1) * 4 * 128);  // [W][128]
-                int32_t* hs = reinterpret_cast<int32_t*>(ks + W * 128);           // [W][128]
                 mbar_expect_tx(&fullc[s], stage_tx);
                 // couplings of block b's rows with the columns of blocks k - L .. k (cyclic in
                 // the sweep; a block before the launch's first is never folded, any rows do)
@@ -499,7 +565,6 @@ __device__ void persist_chain_cta(const SkDev& d, const SkPersistArgs& a, const 
                     tma_load_2d(Jw + i * 4 * 128, &m.jb, b * 128, bi * 4, &fullc[s], pol);
                 }
                 tma_load_2d(ks, &m.kst, b * 128, sw * R + r0, &fullc[s], pol);
-                tma_load_2d(hs, pub ? &m.hpub : &m.h, b * 128, r0, &fullc[s], pol);
                 last_fill[s] = k;
                 return true;
             };
@@ -540,6 +605,40 @@ __device__ void persist_chain_cta(const SkDev& d, const SkPersistArgs& a, const 
                 red_release_add(&D_count[k % Q], 1u);
             }
         }
+    } else if (warp == 2 * W + 2) {
+        // ---------------- fields warp: the fields of block k's rows, once they are published --
+        // (apart from the couplings: those are staged blocks ahead, and the fold warps work on them
+        // while these are still on their way)
+        if (lane == 0) {
+            const uint64_t pol = l2_evict_last();
+            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&m.hpub)) : "memory");
+            int last_fill[kChainStages];
+            for (int s = 0; s < kChainStages; ++s) last_fill[s] = -1;
+            for (int k = 0, b = 0; k < nk; ++k, b = (b + 1 == nb) ? 0 : b + 1) {
+                const int s = k % kChainStages;
+                if (k >= kChainStages && !mbar_wait_or_abort(&emptyc[s], (uint32_t)(k / kChainStages - 1) & 1u,
+                                                             d.err, nowait, abort_flag)) {
+                    atomicOr(d.err, 2048);
+                    *abort_flag = 1;
+                    break;
+                }
+                const bool pub = k > L;
+                if (pub && !wait_at_least(&H_ready[b], (uint32_t)(k + 1), d.err, nowait)) {
+                    atomicOr(d.err, 1024);
+                    *abort_flag = 1;
+                    break;
+                }
+                if (pub) fence_proxy_async_global();  // the fields were written by generic stores
+                uint8_t* hs = ring + (size_t)s * stb + stb - (size_t)W * 128 * 4;
+                mbar_expect_tx(&fullh[s], (uint32_t)(W * 128 * 4));
+                tma_load_2d(hs, pub ? &m.hpub : &m.h, b * 128, r0, &fullh[s], pol);
+                last_fill[s] = k;
+            }
+            if (*abort_flag)  // copies that were issued land before the CTA exits
+                for (int s = 0; s < kChainStages; ++s)
+                    if (last_fill[s] >= 0)
+                        mbar_wait_timed(&fullh[s], (uint32_t)(last_fill[s] / kChainStages) & 1u, kPersistWaitNs);
+        }
     } else if (warp >= W) {
         // ---------------- fold warp of replica w ----------------
         const int w = warp - W;
@@ -549,10 +648,6 @@ __device__ void persist_chain_cta(const SkDev& d, const SkPersistArgs& a, const 
             const int s = k % kChainStages;
             bool ok = mbar_wait_or_abort(&fullc[s], (uint32_t)(k / kChainStages) & 1u, d.err, nowait,
                                          abort_flag);
-            // the chain has finished block k - 2 (its flips and spins are in shared memory)
-            if (ok && k >= 2)
-                ok = mbar_wait_or_abort(&cdone[w * 2 + (k & 1)], (uint32_t)((k - 2) >> 1) & 1u, d.err,
-                                        nowait, abort_flag);
             if (!ok) {
                 if (lane == 0) atomicOr(d.err, 32768);
                 *abort_flag = 1;
@@ -561,15 +656,28 @@ __device__ void persist_chain_cta(const SkDev& d, const SkPersistArgs& a, const 
             const uint32_t* Jw = reinterpret_cast<const uint32_t*>(ring + (size_t)s * stb);
             const int16_t* ks16 = reinterpret_cast<const int16_t*>(Jw + (L + 1) * 4 * 128);
             const int32_t* hs = reinterpret_cast<const int32_t*>(ks16 + W * 128) + w * 128;
+            // blocks k - L .. k - 3 are finished (block k - 1's hand-over waited for k - 3): folded
+            // before the fields arrive, so that this work is not on their way to the chain
             int h[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) h[q] = hs[32 * q + lane];
-#pragma unroll
-            for (int i = 0; i < L - 1; ++i) {
-                int bp = b - L + i;
-                if (bp < 0) bp += nb;  // L < nb
-                fold_block(h, Jw + i * 4 * 128, Fw, Sw, bp, k - L + i >= 0, lane);
+            fold_window<L - 2>(h, Jw, Fw, Sw, b - L, nb, k - L, lane);
+            // the chain has finished block k - 2 (its flips and spins are in shared memory)
+            if (k >= 2)
+                ok = mbar_wait_or_abort(&cdone[w * 2 + (k & 1)], (uint32_t)((k - 2) >> 1) & 1u, d.err,
+                                        nowait, abort_flag);
+            if (ok) {
+                int bp = b - 2;
+                if (bp < 0) bp += nb;
+                fold_block(h, Jw + (L - 2) * 4 * 128, Fw, Sw, bp, k >= 2, lane);
+                ok = mbar_wait_or_abort(&fullh[s], (uint32_t)(k / kChainStages) & 1u, d.err, nowait,
+                                        abort_flag);
             }
+            if (!ok) {
+                if (lane == 0) atomicOr(d.err, 32768);
+                *abort_flag = 1;
+                break;
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) h[q] += hs[32 * q + lane];
             int32_t* hd = hb + ((k & 1) * W + w) * 128;
 #pragma unroll
             for (int q = 0; q < 4; ++q) hd[32 * q + lane] = h[q];
@@ -679,12 +787,12 @@ __device__ void persist_chain_cta(const SkDev& d, const SkPersistArgs& a, const 
 }
 
 template <int W, int L>
-__global__ void __launch_bounds__(32 * (2 * W + 2), 1)
+__global__ void __launch_bounds__(32 * (2 * W + 3), 1)
     k_sk_persist(const __grid_constant__ CUtensorMap mapJ, const __grid_constant__ CUtensorMap mapD,
                  const __grid_constant__ SkPersistMaps maps, SkDev d, SkPersistArgs a) {
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    __shared__ __align__(8) uint64_t bars[2 * kChainStages + 4 * 8];  // chain CTA: W <= 8
+    __shared__ __align__(8) uint64_t bars[3 * kChainStages + 4 * 8];  // chain CTA: W <= 8
     __shared__ uint32_t tslot;
     __shared__ uint32_t done_cnt[8];  // chain CTA: blocks each replica warp has written D for
     __shared__ int abort_flag;
@@ -734,7 +842,7 @@ int sk_persist_fits(const SkDev& d, const SkPersistArgs& a, int num_sms) {
         return 0;
     }
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * (2 * a.W + 2), smem) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * (2 * a.W + 3), smem) !=
         cudaSuccess) {
         cudaGetLastError();
         return 0;
@@ -751,7 +859,7 @@ int sk_persist_sweeps(const SkDev& d, const SkPersistArgs& a, const CUtensorMap&
         return -1;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(a.nG + a.nC));
-    cfg.blockDim = dim3((unsigned)(32 * (2 * a.W + 2)));
+    cfg.blockDim = dim3((unsigned)(32 * (2 * a.W + 3)));
     cfg.dynamicSmemBytes = sk_persist_smem_bytes(d, a);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
