@@ -45,6 +45,10 @@
 // start of every launch.
 #include <cuda.h>
 
+#include <map>
+#include <mutex>
+#include <utility>
+
 #include "sg_internal.cuh"
 #include "sk_internal.cuh"
 
@@ -824,6 +828,24 @@ static void* persist_kernel(int W, int L) {
 
 int sk_persist_lookahead_supported(int L) { return L == 4 || L == 6 || L == 8; }
 
+// The limit is a property of the kernel on a device, shared by every handle and every host thread (the
+// samples of a batch plan their launches one after the other): it only ever grows, under a lock.
+static bool raise_persist_limit(void* kern, int smem) {
+    static std::mutex m;
+    static std::map<std::pair<int, void*>, int> limits;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    std::lock_guard<std::mutex> lock(m);
+    int& limit = limits[{dev, kern}];
+    if (smem <= limit) return true;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    limit = smem;
+    return true;
+}
+
 int sk_persist_fits(const SkDev& d, const SkPersistArgs& a, int num_sms) {
     void* kern = persist_kernel(a.W, a.L);
     // R: whole 32-column chunks of tensor memory, at most one TMA box of spin changes; the
@@ -836,11 +858,7 @@ int sk_persist_fits(const SkDev& d, const SkPersistArgs& a, int num_sms) {
         return 0;
     const size_t smem = sk_persist_smem_bytes(d, a);
     if (smem > 227 * 1024) return 0;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-    }
+    if (!raise_persist_limit(kern, (int)smem)) return 0;
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * (2 * a.W + 3), smem) !=
         cudaSuccess) {
