@@ -126,8 +126,17 @@ void make_map_2d_u16(CUtensorMap* map, const void* base, uint64_t inner, uint64_
 
 class SkModel : public Model {
 public:
-    // prefer few CTAs per persistent launch (set before attach by a batch)
-    void set_compact(bool c) { compact_ = c; }
+    // the split of the persistent launch to try first (set before attach by a batch)
+    void set_split(int W, int TPC) {
+        want_W_ = W;
+        want_TPC_ = TPC;
+    }
+    // blocks of a persistent sweep, or 0 where there is none
+    int persist_blocks() const {
+        const int nb = Np_ / 128;
+        return kernel_ == SG_SK_BLOCKED && (autotune_ || B_ == 128) && R >= 32 && R <= 256 && R % 32 == 0 && nb > 4
+                   ? nb : 0;
+    }
 
     SkModel(int n, const int8_t* J, int n_replicas, const double* temps, uint64_t seed, int kernel,
             int block, const std::vector<int64_t>& tw_, const std::vector<int64_t>& tm_) {
@@ -478,14 +487,13 @@ private:
         a.L = L;
         a.n_sweeps = 1;
         a.Q = kPersistSlots;
-        // alone: the smallest TPC and W whose CTAs all fit (the field work spread widest); in a
-        // batch (compact_): the largest, so that more samples' launches run side by side
-        const int Ws[2] = {compact_ ? 8 : 4, compact_ ? 4 : 8};
-        const int TPCs[3] = {compact_ ? 4 : 1, 2, compact_ ? 1 : 4};
-        for (int W : Ws) {
-            if (R % W) continue;
-            for (int TPC : TPCs) {
-                if (TPC * R > 512) continue;
+        // the split a batch asks for, then the smallest W and TPC whose CTAs all fit (the field work
+        // spread widest)
+        const int splits[7][2] = {{want_W_, want_TPC_}, {4, 1}, {4, 2}, {4, 4}, {8, 1}, {8, 2}, {8, 4}};
+        for (const auto& wt : splits) {
+            const int W = wt[0], TPC = wt[1];
+            if (W == 0 || R % W || TPC * R > 512) continue;
+            {
                 a.W = W;
                 a.nC = R / W;
                 a.TPC = TPC;
@@ -547,7 +555,8 @@ private:
         d_.test_nowait = nowait;
     }
 
-    // Autotuner: time two sweeps with each block size that divides Np and keep the fastest.
+    // Autotuner: time two sweeps (eight where they share one launch, whose start they then hardly
+    // count) with each block size that divides Np and keep the fastest.
     // The trial sweeps run from a fresh state which init_state() then rebuilds, so the choice
     // never changes the trajectory (every block size gives the same integers).
     void tune_block(cudaStream_t st) {
@@ -563,11 +572,13 @@ private:
             check_cuda(cudaMemsetAsync(clock_dev, 0, 4, st), "memset");
             sweep(0, st);  // warm-up
             check_cuda(cudaEventRecord(e0, st), "cudaEventRecord");
-            sweep_many(1, 2, st);  // as the replayed graphs run them
+            const int n = persist_ ? 8 : 2;
+            sweep_many(1, n, st);  // as the replayed graphs run them
             check_cuda(cudaEventRecord(e1, st), "cudaEventRecord");
             check_cuda(cudaEventSynchronize(e1), "cudaEventSynchronize");
             float ms = 0.f;
             check_cuda(cudaEventElapsedTime(&ms, e0, e1), "cudaEventElapsedTime");
+            ms /= (float)n;
             if (best_ms == 0.f || ms < best_ms) {
                 best_ms = ms;
                 best = B;
@@ -632,7 +643,7 @@ private:
     static constexpr int kPersistSlots = kSkPersistSlots;  // spin-change ring slots
     int kernel_ = SG_SK_BLOCKED;
     bool autotune_ = false;
-    bool compact_ = false;
+    int want_W_ = 0, want_TPC_ = 0;
     bool persist_ = false;   // B = 128 sweeps run as one persistent launch
     SkPersistArgs pa_{};
     CUtensorMap mapDr_{};
@@ -698,10 +709,6 @@ public:
             const sg_sk_sample& x = samples[b];
             try {
                 subs_.emplace_back(new SkModel(x.n, x.J, n_replicas, x.temps, x.seed, kernel, block, tw, tm));
-                // the samples' persistent launches share the GPU: few CTAs each
-                // (SG_SK_BATCH_COMPACT=0: each as if alone; the results are the same)
-                const char* c = getenv("SG_SK_BATCH_COMPACT");
-                subs_.back()->set_compact(!(c && c[0] == '0' && !c[1]));
             } catch (const Error& e) {
                 fail(e.code, "sample " + std::to_string(b) + ": " + e.msg);
             }
@@ -722,6 +729,7 @@ public:
 
     void attach(char* ws, cudaStream_t st) override {
         clock_dev = reinterpret_cast<uint32_t*>(ws);
+        plan_splits();
         size_t off = 256;
         for (auto& m : subs_) {
             off = (off + 255) & ~size_t(255);
@@ -744,10 +752,10 @@ public:
 
     void sweep(uint32_t t_off, cudaStream_t st) override { sweep_many(t_off, 1, st); }
 
-    // every sample's n sweeps on its own branch, joined once
+    // every sample's n sweeps on its own branch, joined once; the longest first
     void sweep_many(uint32_t t_off, int n, cudaStream_t st) override {
         check_cuda(cudaEventRecord(fork_, st), "cudaEventRecord");
-        for (size_t b = 0; b < subs_.size(); ++b) {
+        for (size_t b : order_) {
             check_cuda(cudaStreamWaitEvent(streams_[b], fork_, 0), "cudaStreamWaitEvent");
             subs_[b]->sweep_many(t_off, n, streams_[b]);
             check_cuda(cudaEventRecord(events_[b], streams_[b]), "cudaEventRecord");
@@ -849,6 +857,79 @@ public:
     }
 
 private:
+    // The samples' persistent launches share the GPU, each resident as a whole: a wide split ends
+    // sooner but leaves less room.  Start from few CTAs each (8 replicas a chain CTA, 2 tiles a field
+    // CTA), look at which sample ends last when the longest go first and the others follow as CTAs
+    // fall free, and widen that one until the end would come later.  us a sweep of the batch, as few CTAs
+    // as possible for every sample, in their own order -> now: 8 samples of N = 2^9 .. 2^12.5, 128
+    // replicas 102 -> 71; 3 of 2^9 .. 2^11, 64 replicas 30 -> 19; 24 of 2^9 .. 2^12 160 -> 129.  Only the ratios of the times count:
+    // us a block, 128 replicas, N = 5000, for (W, TPC) = (4, 1) 1.31, (4, 2) 1.56, (8, 2) 1.79 ((8, 4) 2.07:
+    // its field CTAs read 80 KB a block).
+    void plan_splits() {
+        struct Split { int W, TPC; double us; };
+        static const Split kSplits[3] = {{8, 2, 1.79}, {4, 2, 1.56}, {4, 1, 1.31}};
+        const size_t n = subs_.size();
+        std::vector<int> split(n, 0);
+        order_.resize(n);
+        for (size_t b = 0; b < n; ++b) order_[b] = b;
+        // SG_SK_BATCH_COMPACT=0: each as if alone (the results are the same)
+        const char* c = getenv("SG_SK_BATCH_COMPACT");
+        if (c && c[0] == '0' && !c[1]) return;
+        int dev = 0, sms = 0;
+        check_cuda(cudaGetDevice(&dev), "cudaGetDevice");
+        check_cuda(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev), "cudaDeviceGetAttribute");
+        auto ctas = [&](size_t b) {
+            const Split& s = kSplits[split[b]];
+            const int nb = subs_[b]->persist_blocks();
+            return R / s.W + (nb + s.TPC - 1) / s.TPC;
+        };
+        auto time = [&](size_t b) { return subs_[b]->persist_blocks() * kSplits[split[b]].us; };
+        auto last_to_end = [&](double& end) {  // longest first, each as soon as its CTAs are free
+            std::stable_sort(order_.begin(), order_.end(), [&](size_t x, size_t y) { return time(x) > time(y); });
+            std::vector<size_t> waiting(order_), running;
+            std::vector<double> ends(n, 0.0);
+            double now = 0.0;
+            int used = 0;
+            size_t last = order_[0];
+            end = 0.0;
+            while (!waiting.empty() || !running.empty()) {
+                for (auto it = waiting.begin(); it != waiting.end();) {
+                    if (used + ctas(*it) <= sms || running.empty()) {
+                        used += ctas(*it);
+                        ends[*it] = now + time(*it);
+                        running.push_back(*it);
+                        it = waiting.erase(it);
+                    } else {
+                        ++it;
+                    }
+                }
+                auto next = std::min_element(running.begin(), running.end(),
+                                             [&](size_t x, size_t y) { return ends[x] < ends[y]; });
+                now = ends[*next];
+                if (now >= end) {
+                    end = now;
+                    last = *next;
+                }
+                used -= ctas(*next);
+                running.erase(next);
+            }
+            return last;
+        };
+        double end;
+        size_t last = last_to_end(end);
+        while (split[last] < 2) {
+            const size_t b = last;
+            const double before = end;
+            ++split[b];
+            last = last_to_end(end);
+            if (end <= before && ctas(b) <= sms) continue;  // as soon: another may end with it
+            --split[b];
+            last_to_end(end);
+            break;
+        }
+        for (size_t b = 0; b < n; ++b) subs_[b]->set_split(kSplits[split[b]].W, kSplits[split[b]].TPC);
+    }
+
     void collect() {
         for (auto& m : subs_) {
             launches += m->launches;
@@ -869,6 +950,7 @@ private:
     std::vector<cudaStream_t> streams_;
     std::vector<cudaEvent_t> events_;
     cudaEvent_t fork_ = nullptr;
+    std::vector<size_t> order_;  // the samples in launch order
 };
 
 }  // namespace
