@@ -15,8 +15,8 @@
 // of N = 2^22 (degree 4, two replicas) reads 84 bytes per vertex from HBM (31 % of its peak), gathers
 // 16.8 million word pairs, each a 32-byte sector of L2 (45 %) and a tag of L1 (50 %), and issues 515
 // instructions per slice (41 %).  us a sweep, before (groups staged by bulk copies into shared-memory
-// rings, a launch per sweep) -> now: N = 2^22 131 -> 128, 2^20 50 -> 39, bipartite 2^18 14.2 -> 10.3,
-// N = 300007 with one replica (a launch per class) 30.8 -> 17, N = 20011 with four 23.3 -> 18.3.
+// rings, a launch per sweep) -> now: N = 2^22 131 -> 128, 2^20 50 -> 39, bipartite 2^18 14.2 -> 9.6,
+// N = 300007 with one replica (a launch per class) 30.8 -> 16, N = 20011 with four 24.9 -> 16.1.
 // Without the rings there is no pipeline to fill and drain in each class, and no launch gap.
 #include <algorithm>
 
@@ -28,10 +28,12 @@ namespace sg {
 
 namespace {
 
-// threads of a CTA (two CTAs share an SM) and entries per chunk
+// threads of a CTA (two CTAs share an SM) and entries per chunk; four replicas with chunks of 8 need
+// 255 registers (128 threads: N = 20011 16.1 us a sweep, N = 10^5 23.3; 192 threads with spills 17.4,
+// 25.9)
 template <int R, int CH>
 struct SweepShape {
-    static constexpr int threads = CH == 8 ? (R == 4 ? 192 : 256) : R == 1 ? 384 : R == 2 ? 320 : 256;
+    static constexpr int threads = CH == 8 ? (R == 4 ? 128 : 256) : R == 1 ? 384 : R == 2 ? 320 : 256;
 };
 
 constexpr int kSweepTables = 16;  // graphs whose thresholds are kept in shared memory
@@ -87,9 +89,9 @@ __device__ __forceinline__ void accept_from(uint32_t vi, uint32_t t, uint64_t se
     }
 }
 
-__device__ __forceinline__ uint32_t ld_relaxed_u32(const uint32_t* p) {
+__device__ __forceinline__ uint32_t ld_acquire_u32(const uint32_t* p) {
     uint32_t v;
-    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
 
@@ -110,7 +112,7 @@ __global__ void __launch_bounds__(SweepShape<R, kChunk>::threads, 2)
     const uint32_t tid = threadIdx.x, lane = tid & 31u;
     const uint32_t nc = (uint32_t)d.n_colours;
     const uint32_t gw = (tid >> 5) * gridDim.x + blockIdx.x;  // neighbouring slices on different SMs
-    const uint32_t stride = (blockDim.x >> 5) * gridDim.x;  // at least a CTA's warps: one round in the tail
+    const uint32_t stride = (blockDim.x >> 5) * gridDim.x;
     for (uint32_t i = tid; i <= nc; i += blockDim.x) cs[i] = __ldg(d.class_slice + i);
     const bool tables = d.n_graphs <= kSweepTables;
     if (tables) {
@@ -125,8 +127,9 @@ __global__ void __launch_bounds__(SweepShape<R, kChunk>::threads, 2)
     const uint64_t pol_stream = d.stream_first ? l2_evict_first() : pol_keep;
 
     // move to the warp's next slice, if there is one (sweep == n_sweeps: none)
-    // the thin classes at the end, each at most one slice per warp of a CTA, are all the first CTA's:
-    // they need no grid-wide barrier between them
+    // The thin classes at the end, each at most one slice per warp of a CTA, are all the first CTA's:
+    // they need no grid-wide barrier between them (two or three rounds there take longer than a
+    // barrier: N = 10^5, R = 2 18.3 us a sweep against 16.4).
     const uint32_t warps = blockDim.x >> 5;
     uint32_t tail = nc;
     while (tail > 0 && cs[tail] - cs[tail - 1] <= warps) --tail;
@@ -152,8 +155,11 @@ __global__ void __launch_bounds__(SweepShape<R, kChunk>::threads, 2)
     settle(nx);
     uint4 nm = load_meta(nx);
     Cursor nn = nx;  // the one after, of which only the meta data is read ahead
-    nn.slice += stride;
-    settle(nn);
+    auto step = [&](Cursor& c) {
+        c.slice += c.cls < tail ? stride : warps;
+        settle(c);
+    };
+    step(nn);
     uint4 nnm = load_meta(nn);
     auto load_vi = [&](const Cursor& c) -> uint32_t {
         return c.sweep < n_sweeps ? ld_stream_u32(d.vinfo + (int64_t)c.slice * 32 + lane, pol_stream) : kInactive;
@@ -202,22 +208,24 @@ __global__ void __launch_bounds__(SweepShape<R, kChunk>::threads, 2)
     for (uint32_t q = 0; q < nq; ++q) {
         if (nx.sweep == sweep && nx.cls == cls) next_acceptance();
         if (phase > 0 && cls <= tail && gridDim.x > 1) {
-            // admitted once every CTA has written the classes before (bounded; the polls are relaxed
-            // loads and one fence: an acquire in each would drop the L1 each time)
+            // admitted once every CTA has written the classes before (bounded).  Acquiring polls: the
+            // words are read from L2 and the tables from shared memory, so nothing is lost with the L1,
+            // and a fence after relaxed polls costs 0.3 to 0.4 us more (of 2.2 us between two classes
+            // that hold one gather and one store, 152 CTAs; flags polled by every CTA 6.5, eight
+            // counters 2.3).
             if (tid == 0) {
                 const uint32_t target = phase * gridDim.x;
-                int pass = ld_relaxed_u32(d.gbar) >= target;
+                int pass = ld_acquire_u32(d.gbar) >= target;
                 if (!pass && d.stage_wait_ns) {
                     const uint64_t ns0 = global_ns();
                     for (uint32_t it = 1;; ++it) {
-                        if (ld_relaxed_u32(d.gbar) >= target) {
+                        if (ld_acquire_u32(d.gbar) >= target) {
                             pass = 1;
                             break;
                         }
                         if ((it & 255u) == 0u && global_ns() - ns0 > d.stage_wait_ns) break;
                     }
                 }
-                asm volatile("fence.acq_rel.gpu;" ::: "memory");
                 if (!pass) {
                     atomicOr(d.err, 8);
                     s_ok = 0;
@@ -238,8 +246,7 @@ __global__ void __launch_bounds__(SweepShape<R, kChunk>::threads, 2)
                 nx = nn;
                 nm = nnm;
                 nvi = nnvi;
-                nn.slice += stride;
-                settle(nn);
+                step(nn);
                 load_slice();
                 nnm = load_meta(nn);
                 nnvi = load_vi(nn);
@@ -358,7 +365,7 @@ static int launch_sweeps(const VbPackedDev& d, int max_class_slices, int sms, ui
 
 // Chunks of 8 entries where every warp has at most one slice of a class: the class then takes as long
 // as its widest slice, and fewer rounds of gathers count for more than warps in flight (R = 2,
-// N = 65536: 15.6 us a sweep, 16.6 with chunks of 4; R = 4, N = 60000: 24.6, 27.1).  Beyond that the
+// N = 65536: 15.6 us a sweep, 16.6 with chunks of 4; R = 4, N = 60000: 23.3, 27.1).  Beyond that the
 // registers are better spent on more warps (R = 2, bipartite N = 2^18: 10.3 us with chunks of 4,
 // 11.9 with 8; Poissonian N = 2^22: 128, 145; R = 4, N = 10^6: 80, 90).
 template <int R>
