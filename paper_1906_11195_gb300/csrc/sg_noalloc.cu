@@ -36,34 +36,87 @@ __device__ __forceinline__ uint32_t e4m3_signs(uint32_t v) {
     return nz * 0x38u | neg;
 }
 
-// bytes [o, o + 16) of a row of n, as four words; those at or past n are zero.  `row` starts at byte
-// `off` of the array [a, a + len); only whole 4-byte words inside the array are read as words.
-__device__ __forceinline__ uint4 load_row16(const int8_t* __restrict__ a, int64_t len, int64_t off,
-                                            int o, int n) {
-    uint32_t w[4] = {0u, 0u, 0u, 0u};
-    if (o < n) {
-        const int8_t* p = a + off + o;
-        const int m = n - o < 16 ? n - o : 16;
-        if (((uintptr_t)p & 15u) == 0 && m == 16) {
-            return __ldg(reinterpret_cast<const uint4*>(p));
-        }
-        const uint32_t sh = ((uintptr_t)p & 3u) * 8u;
+// 16 bytes of a row from p, of which m are the row's (the rest becomes zero).  Words holds what is loaded
+// ahead: with A16 the piece itself (p 16-byte aligned, m = 16), else the five 4-byte words around it,
+// where all of them lie inside the array [a, end); otherwise finish() reads the bytes one by one.
+template <bool A16>
+struct Piece {
+    uint32_t x[A16 ? 4 : 5];
+    const int8_t* p;
+    int m;
+    __device__ __forceinline__ bool words(const int8_t* a, const int8_t* end) const {
         const int8_t* q = p - ((uintptr_t)p & 3u);
-        if (q >= a && q + 20 <= a + len) {
-            uint32_t x[5];
+        return q >= a && q + 20 <= end;
+    }
+    __device__ __forceinline__ void load(const int8_t* a, const int8_t* end) {
+        if constexpr (A16) {
+            const uint4 v = m > 0 ? __ldg(reinterpret_cast<const uint4*>(p)) : make_uint4(0u, 0u, 0u, 0u);
+            x[0] = v.x;
+            x[1] = v.y;
+            x[2] = v.z;
+            x[3] = v.w;
+        } else {
+            const bool in = m > 0 && words(a, end);
+            const uint32_t* q = reinterpret_cast<const uint32_t*>(p - ((uintptr_t)p & 3u));
 #pragma unroll
-            for (int k = 0; k < 5; ++k) x[k] = __ldg(reinterpret_cast<const uint32_t*>(q) + k);
+            for (int k = 0; k < 5; ++k) x[k] = in ? __ldg(q + k) : 0u;
+        }
+    }
+    __device__ __forceinline__ uint4 finish(const int8_t* a, const int8_t* end) const {
+        if constexpr (A16) return make_uint4(x[0], x[1], x[2], x[3]);
+        uint32_t w[4] = {0u, 0u, 0u, 0u};
+        if (m > 0 && !words(a, end)) {
+            for (int k = 0; k < m; ++k) w[k >> 2] |= (uint32_t)(uint8_t)__ldg(p + k) << (8 * (k & 3));
+        } else if (m > 0) {
+            const uint32_t sh = ((uintptr_t)p & 3u) * 8u;
 #pragma unroll
-            for (int k = 0; k < 4; ++k) w[k] = __funnelshift_r(x[k], x[k + 1], sh);
-            for (int k = 0; k < 4; ++k) {  // beyond the row
+            for (int k = 0; k < 4; ++k) {
+                w[k] = __funnelshift_r(x[k], x[k + 1 < 5 ? k + 1 : 4], sh);
                 const int left = m - 4 * k;
                 if (left < 4) w[k] = left <= 0 ? 0u : w[k] & ((1u << (8 * left)) - 1u);
             }
-        } else {
-            for (int k = 0; k < m; ++k) w[k >> 2] |= (uint32_t)(uint8_t)__ldg(p + k) << (8 * (k & 3));
+        }
+        return make_uint4(w[0], w[1], w[2], w[3]);
+    }
+};
+
+// The CTA's operands into shared memory: 16-byte pieces of kt tiles of 128 columns from k0 of the
+// coupling rows m0 .. m0 + 127 and of the R spin rows; piece c of row r goes to c ^ (r & 7) of that row.
+// Several pieces of a thread are on their way at once.
+template <bool A16>
+__device__ __forceinline__ void load_operands(const int8_t* __restrict__ J, const int8_t* __restrict__ s,
+                                              int n, int R, int kt, int m0, int k0, uint8_t* sA,
+                                              uint8_t* sB, int tid) {
+    constexpr int U = A16 ? 8 : 4;
+    const int pieces = kt * 8, lp = kt == 2 ? 4 : 3;  // kt is 1 or 2
+    const int total = (128 + R) * pieces;
+    const int8_t *end_j = J + (int64_t)n * n, *end_s = s + (int64_t)R * n;
+    for (int i0 = tid; i0 < total; i0 += kFieldsThreads * U) {
+        Piece<A16> pc[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int i = i0 + u * kFieldsThreads, row = i >> lp, o = k0 + (i & (pieces - 1)) * 16;
+            const bool j = row < 128;
+            const int left = n - o;
+            pc[u].m = i < total && (!j || m0 + row < n) ? (left < 16 ? left : 16) : 0;
+            pc[u].p = j ? J + (int64_t)(m0 + row) * n + o : s + (int64_t)(row - 128) * n + o;
+            pc[u].load(j ? J : s, j ? end_j : end_s);
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int i = i0 + u * kFieldsThreads, row = i >> lp, c = i & (pieces - 1);
+            if (i >= total) break;
+            const bool j = row < 128;
+            const int r = j ? row : row - 128;
+            uint4 v = pc[u].finish(j ? J : s, j ? end_j : end_s);
+            v.x = e4m3_signs(v.x);
+            v.y = e4m3_signs(v.y);
+            v.z = e4m3_signs(v.z);
+            v.w = e4m3_signs(v.w);
+            uint8_t* tile = j ? sA + (size_t)(c >> 3) * 128 * 128 : sB + (size_t)(c >> 3) * R * 128;
+            *reinterpret_cast<uint4*>(tile + r * 128 + (((c & 7) ^ (r & 7)) << 4)) = v;
         }
     }
-    return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
 __device__ __forceinline__ uint32_t fields_rank() {
@@ -111,29 +164,10 @@ __global__ void __launch_bounds__(kFieldsThreads)
         mbar_init(&bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    // 16-byte pieces of both operands: piece c of row r goes to c ^ (r & 7) of that row
-    const int pieces = kt * 8, lp = kt == 2 ? 4 : 3;  // kt is 1 or 2
-    const int64_t len_j = (int64_t)n * n, len_s = (int64_t)R * n;
-#pragma unroll 8
-    for (int i = tid; i < (128 + R) * pieces; i += kFieldsThreads) {
-        const int row = i >> lp, c = i & (pieces - 1);
-        const int o = k0 + c * 16;
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        uint8_t* dst;
-        if (row < 128) {
-            if (m0 + row < n) v = load_row16(J, len_j, (int64_t)(m0 + row) * n, o, n);
-            dst = sA + (size_t)(c >> 3) * 128 * 128 + row * 128 + (((c & 7) ^ (row & 7)) << 4);
-        } else {
-            const int r = row - 128;
-            v = load_row16(s, len_s, (int64_t)r * n, o, n);
-            dst = sB + (size_t)(c >> 3) * R * 128 + r * 128 + (((c & 7) ^ (r & 7)) << 4);
-        }
-        v.x = e4m3_signs(v.x);
-        v.y = e4m3_signs(v.y);
-        v.z = e4m3_signs(v.z);
-        v.w = e4m3_signs(v.w);
-        *reinterpret_cast<uint4*>(dst) = v;
-    }
+    if ((((uintptr_t)J | (uintptr_t)s | (uintptr_t)n) & 15u) == 0)
+        load_operands<true>(J, s, n, R, kt, m0, k0, sA, sB, tid);
+    else
+        load_operands<false>(J, s, n, R, kt, m0, k0, sA, sB, tid);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
