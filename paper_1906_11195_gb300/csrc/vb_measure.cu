@@ -14,6 +14,8 @@
 // and a 32-byte sector per gathered word), on small ones the latency of one run.  The run length
 // therefore follows the size: as many warps as the GPU holds, up to kMeasureRun rows each (the
 // sum over the 32 threads costs about as much as 30 rows' additions).
+#include <algorithm>
+
 #include "../../include/sg.h"
 #include "sg_internal.cuh"
 #include "vb_bits.cuh"
@@ -222,19 +224,27 @@ int vb_packed_measure(const VbPackedDev& d, const VbMeasure& m, cudaStream_t st)
     if (rows == 0) return 0;
     MeasureGrid mg;
     mg.up_rows = d.up_rows;
-    // whole waves of the CTAs that the 152 SMs hold at once, a run as long as that allows
+    // Whole waves of the CTAs that the 152 SMs hold at once.  In one or two waves the slowest run is the
+    // time: a row of edges takes longer than a row of spins (its gathers wait for its slots), so its
+    // runs are half as long (five snapshots, N = 2^20: 72 -> 60 us; a third as long 61, a quarter 65).
+    // More waves even out by themselves (N = 2^22: 180 us, with shorter edge runs 185).
     const int64_t slots = 152 * (d.R == 4 ? kMeasureCtas<4> : kMeasureCtas<2>);
-    const int64_t waves = (rows + slots * kMeasureWarps * kMeasureRun - 1) / (slots * kMeasureWarps * kMeasureRun);
-    int64_t run = (rows + waves * slots * kMeasureWarps - 1) / (waves * slots * kMeasureWarps);
+    auto waves_of = [&](int64_t c) { return (c + slots * kMeasureWarps * kMeasureRun - 1) / (slots * kMeasureWarps * kMeasureRun); };
+    const int64_t edge_cost = waves_of(rows) <= 2 ? 2 : 1;
+    const int64_t cost = (int64_t)d.n_slices * passes + (m.e ? (int64_t)d.up_rows * edge_cost : 0);
+    const int64_t waves = waves_of(cost);
+    int64_t run = (cost + waves * slots * kMeasureWarps - 1) / (waves * slots * kMeasureWarps);
+    auto edge_run = [&](int64_t r) { return std::max<int64_t>(1, r / edge_cost); };
     auto ctas = [&](int64_t r) {  // each pass's last CTA is part empty
-        const int64_t n = r * kMeasureWarps;
-        return (d.n_slices + n - 1) / n * passes + (m.e ? ((int64_t)d.up_rows + n - 1) / n : 0);
+        const int64_t n = r * kMeasureWarps, ne = edge_run(r) * kMeasureWarps;
+        return (d.n_slices + n - 1) / n * passes + (m.e ? ((int64_t)d.up_rows + ne - 1) / ne : 0);
     };
     while (run < kMeasureRun && ctas(run) > waves * slots) ++run;
-    mg.run_s = mg.run_e = (int)run;
-    const int64_t per_cta = run * kMeasureWarps;
+    mg.run_s = (int)run;
+    mg.run_e = (int)edge_run(run);
+    const int64_t per_cta = run * kMeasureWarps, per_cta_e = mg.run_e * kMeasureWarps;
     mg.nb_s = passes ? (uint32_t)((d.n_slices + per_cta - 1) / per_cta) : 1u;
-    mg.nb_e = m.e ? (uint32_t)(((int64_t)d.up_rows + per_cta - 1) / per_cta) : 0u;
+    mg.nb_e = m.e ? (uint32_t)(((int64_t)d.up_rows + per_cta_e - 1) / per_cta_e) : 0u;
     const int64_t nb = (int64_t)mg.nb_e + (int64_t)mg.nb_s * passes;
     if (nb > 0x7FFFFFFF) return -1;
     switch (d.R) {
