@@ -28,6 +28,8 @@ void check_cuda(cudaError_t e, const char* what);
 // Page-locked host memory for the large host-side images that sg_attach copies to the device
 // (so the copies run at DMA speed); plain heap memory where no CUDA device is present.  A
 // 64-byte header before each block records which of the two it came from.
+// Page-locking and unlocking a block takes longer than copying a small one from pageable memory.
+constexpr size_t kPinnedMin = (size_t)1 << 20;
 template <class T>
 struct PinnedAllocator {
     using value_type = T;
@@ -37,9 +39,9 @@ struct PinnedAllocator {
     T* allocate(size_t n) {
         const size_t bytes = n * sizeof(T) + 64;
         void* p = nullptr;
-        int pinned = 1;
-        if (cudaMallocHost(&p, bytes) != cudaSuccess || !p) {
-            cudaGetLastError();
+        int pinned = bytes >= kPinnedMin;
+        if (!pinned || cudaMallocHost(&p, bytes) != cudaSuccess || !p) {
+            if (pinned) cudaGetLastError();
             pinned = 0;
             p = malloc(bytes);
             if (!p) throw std::bad_alloc();

@@ -352,11 +352,8 @@ public:
 
     void read_windows(const int64_t* cnt_c, const int64_t* cnt_q, int64_t* C, int64_t* q,
                       int64_t* E, cudaStream_t st) override {
-        std::vector<int64_t> c(nwC()), qq(nwQ()), e(nwE());
-        down(c.data(), wC_, c.size() * 8, st);
-        down(qq.data(), wQ_, qq.size() * 8, st);
-        down(e.data(), wE_, e.size() * 8, st);
-        check_cuda(cudaStreamSynchronize(st), "read windows");
+        const Counts all = read_counts(wC_, wQ_, wE_, nwE(), st, "read windows");
+        const int64_t *c = all.c, *qq = all.q, *e = all.e;
         const int64_t ntw = (int64_t)tw.size(), nb = n_bins;
         for (int r = 0; r < R; ++r)
             for (int64_t m = 0; m < nb; ++m) {
@@ -373,18 +370,13 @@ public:
         const int64_t ntw = (int64_t)tw.size();
         int active = 0;
         while (active < (int)ntw && tw[active] <= tau) ++active;
-        check_cuda(cudaMemsetAsync(mC_, 0, nmC() * 8, st), "memset");
-        if (nmQ()) check_cuda(cudaMemsetAsync(mQ_, 0, nmQ() * 8, st), "memset");
-        check_cuda(cudaMemsetAsync(mE_, 0, nmE() * 8, st), "memset");
+        check_cuda(cudaMemsetAsync(mC_, 0, (size_t)(mE_ - mC_ + (int64_t)nmE()) * 8, st), "memset");
         launches += sk_measure(d_, active, mC_, ntw, 1, R >= 2 ? mQ_ : nullptr, 1, mE_, 1, st);
     }
 
     void read_scheduled(int64_t tau, int64_t* C, int64_t* q, int64_t* E, cudaStream_t st) override {
-        std::vector<int64_t> c(nC()), qq(nQ()), e(nE());
-        down(c.data(), dC_, c.size() * 8, st);
-        down(qq.data(), dQ_, qq.size() * 8, st);
-        down(e.data(), dE_, e.size() * 8, st);
-        check_cuda(cudaStreamSynchronize(st), "read results");
+        const Counts all = read_counts(dC_, dQ_, dE_, nE(), st, "read results");
+        const int64_t *c = all.c, *qq = all.q, *e = all.e;
         const int64_t ntw = (int64_t)tw.size(), ntm = (int64_t)tm.size();
         for (int r = 0; r < R; ++r)
             for (int64_t u = 0; u < ntm; ++u) {
@@ -399,11 +391,8 @@ public:
     }
 
     void read_now(int64_t tau, int64_t* C, int64_t* q, int64_t* E, cudaStream_t st) override {
-        std::vector<int64_t> c(nmC()), qq(nmQ()), e(nmE());
-        down(c.data(), mC_, c.size() * 8, st);
-        down(qq.data(), mQ_, qq.size() * 8, st);
-        down(e.data(), mE_, e.size() * 8, st);
-        check_cuda(cudaStreamSynchronize(st), "read measurement");
+        const Counts all = read_counts(mC_, mQ_, mE_, nmE(), st, "read measurement");
+        const int64_t *c = all.c, *qq = all.q, *e = all.e;
         const int64_t ntw = (int64_t)tw.size();
         for (int r = 0; r < R; ++r) {
             for (int64_t w = 0; w < ntw; ++w)
@@ -456,6 +445,23 @@ private:
     size_t nwC() const { return (size_t)R * tw.size() * n_bins; }
     size_t nwQ() const { return (size_t)(R / 2) * n_bins; }
     size_t nwE() const { return (size_t)R * n_bins; }
+
+    // C, q and E counts, which lie one after the other in the workspace, in one copy
+    struct Counts {
+        std::vector<int64_t> buf;
+        const int64_t *c, *q, *e;
+    };
+    Counts read_counts(const int64_t* c, const int64_t* q, const int64_t* e, size_t n_e,
+                       cudaStream_t st, const char* what) {
+        Counts r;
+        r.buf.resize((size_t)(e - c) + n_e);
+        down(r.buf.data(), c, r.buf.size() * 8, st);
+        check_cuda(cudaStreamSynchronize(st), what);
+        r.c = r.buf.data();
+        r.q = r.c + (q - c);
+        r.e = r.c + (e - c);
+        return r;
+    }
 
     void down(void* dst, const void* src, size_t bytes, cudaStream_t st) {
         d2h_bytes += (int64_t)bytes;
