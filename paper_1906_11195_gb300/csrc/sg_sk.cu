@@ -864,18 +864,18 @@ public:
 
 private:
     // The samples' persistent launches share the GPU, each resident as a whole: a wide split ends
-    // sooner but leaves less room.  Start from few CTAs each (8 replicas a chain CTA, 2 tiles a field
-    // CTA), look at which sample ends last when the longest go first and the others follow as CTAs
-    // fall free, and widen that one until the end would come later.  us a sweep of the batch, as few CTAs
-    // as possible for every sample, in their own order -> now: 8 samples of N = 2^9 .. 2^12.5, 128
-    // replicas 102 -> 71; 3 of 2^9 .. 2^11, 64 replicas 30 -> 19; 24 of 2^9 .. 2^12 160 -> 129.  Only the ratios of the times count:
-    // us a block, 128 replicas, N = 5000, for (W, TPC) = (4, 1) 1.31, (4, 2) 1.56, (8, 2) 1.79 ((8, 4) 2.07:
-    // its field CTAs read 80 KB a block).
+    // sooner but leaves less room.  Start from as few CTAs as possible (8 replicas a chain CTA, 4 tiles a
+    // field CTA), look at which sample ends last when the longest go first and the others follow as
+    // CTAs fall free, and widen that one until the end would come later.  Only the ratios of the times
+    // count: us a block, 128 replicas, N = 5000, for (W, TPC) = (8, 4) 2.07, (8, 2) 1.79, (4, 2) 1.56,
+    // (4, 1) 1.31.  us a sweep of the batch, all (8, 4) in their own order -> now: 8 samples of N = 2^9 ..
+    // 2^12.5, 128 replicas 102 -> 71; 3 of 2^9 .. 2^11, 64 replicas 30 -> 21; 24 of 2^9 .. 2^12 160 -> 136;
+    // 32 of 2^9 .. 2^14 0.80 ms -> 0.75.
     void plan_splits() {
         struct Split { int W, TPC; double us; };
-        static const Split kSplits[3] = {{8, 2, 1.79}, {4, 2, 1.56}, {4, 1, 1.31}};
+        static const Split kSplits[4] = {{8, 4, 2.07}, {8, 2, 1.79}, {4, 2, 1.56}, {4, 1, 1.31}};
         const size_t n = subs_.size();
-        std::vector<int> split(n, 0);
+        std::vector<int> split(n, 4 * R <= 512 ? 0 : 1);  // 512 columns of tensor memory
         order_.resize(n);
         for (size_t b = 0; b < n; ++b) order_[b] = b;
         // SG_SK_BATCH_COMPACT=0: each as if alone (the results are the same)
@@ -923,7 +923,7 @@ private:
         };
         double end;
         size_t last = last_to_end(end);
-        while (split[last] < 2) {
+        while (split[last] < 3) {
             const size_t b = last;
             const double before = end;
             ++split[b];
