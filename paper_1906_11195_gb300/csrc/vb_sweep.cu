@@ -36,7 +36,7 @@ struct SweepShape {
     static constexpr int threads = CH == 8 ? (R == 4 ? 128 : 256) : R == 1 ? 384 : R == 2 ? 320 : 256;
 };
 
-constexpr int kSweepTables = 16;  // graphs whose thresholds are kept in shared memory
+constexpr int kSweepTables = 32;  // graphs whose thresholds are kept in shared memory
 constexpr int kSweepPlanes = 4;  // counter planes: slices up to width 15; wider ones count apart
 
 __device__ __forceinline__ uint32_t ld_stream_u32(const uint32_t* p, uint64_t pol) {
