@@ -50,6 +50,7 @@
 #include <utility>
 
 #include "sg_internal.cuh"
+#include "sk_fields_warp.h"
 #include "sk_internal.cuh"
 
 namespace sg {
@@ -58,7 +59,6 @@ namespace {
 
 constexpr uint64_t kPersistWaitNs = 2000000000ull;  // 2 s: only a broken launch waits that long
 constexpr uint32_t kTileBytes = 128 * 128;          // one e4m3 128 x 128 coupling tile
-constexpr int kChainStages = 3;  // staged blocks ahead of the chain
 
 __device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
     uint32_t v;
@@ -616,32 +616,37 @@ __device__ void persist_chain_cta(const SkDev& d, const SkPersistArgs& a, const 
         if (lane == 0) {
             const uint64_t pol = l2_evict_last();
             asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&m.hpub)) : "memory");
-            int last_fill[kChainStages];
-            for (int s = 0; s < kChainStages; ++s) last_fill[s] = -1;
-            for (int k = 0, b = 0; k < nk; ++k, b = (b + 1 == nb) ? 0 : b + 1) {
-                const int s = k % kChainStages;
-                if (k >= kChainStages && !mbar_wait_or_abort(&emptyc[s], (uint32_t)(k / kChainStages - 1) & 1u,
-                                                             d.err, nowait, abort_flag)) {
-                    atomicOr(d.err, 2048);
+            struct Ops {
+                const SkDev& d;
+                const SkPersistMaps& m;
+                uint8_t* ring;
+                uint64_t *emptyc, *fullh;
+                const uint32_t* H_ready;
+                volatile int* abort_flag;
+                size_t stb;
+                uint64_t pol;
+                int r0;
+                bool nowait;
+                __device__ bool give_up(int bit) {
+                    atomicOr(d.err, bit);
                     *abort_flag = 1;
-                    break;
+                    return false;
                 }
-                const bool pub = k > L;
-                if (pub && !wait_at_least(&H_ready[b], (uint32_t)(k + 1), d.err, nowait)) {
-                    atomicOr(d.err, 1024);
-                    *abort_flag = 1;
-                    break;
+                __device__ bool wait_empty(int s, uint32_t phase) {
+                    return mbar_wait_or_abort(&emptyc[s], phase, d.err, nowait, abort_flag) || give_up(2048);
                 }
-                if (pub) fence_proxy_async_global();  // the fields were written by generic stores
-                uint8_t* hs = ring + (size_t)s * stb + stb - (size_t)W * 128 * 4;
-                mbar_expect_tx(&fullh[s], (uint32_t)(W * 128 * 4));
-                tma_load_2d(hs, pub ? &m.hpub : &m.h, b * 128, r0, &fullh[s], pol);
-                last_fill[s] = k;
-            }
-            if (*abort_flag)  // copies that were issued land before the CTA exits
-                for (int s = 0; s < kChainStages; ++s)
-                    if (last_fill[s] >= 0)
-                        mbar_wait_timed(&fullh[s], (uint32_t)(last_fill[s] / kChainStages) & 1u, kPersistWaitNs);
+                __device__ bool wait_published(int b, int k) {
+                    return wait_at_least(&H_ready[b], (uint32_t)(k + 1), d.err, nowait) || give_up(1024);
+                }
+                __device__ void copy(int s, int b, bool pub) {
+                    if (pub) fence_proxy_async_global();  // the fields were written by generic stores
+                    mbar_expect_tx(&fullh[s], (uint32_t)(W * 128 * 4));
+                    tma_load_2d(ring + (size_t)s * stb + stb - (size_t)W * 128 * 4, pub ? &m.hpub : &m.h,
+                                b * 128, r0, &fullh[s], pol);
+                }
+                __device__ void drain(int s, uint32_t phase) { mbar_wait_timed(&fullh[s], phase, kPersistWaitNs); }
+            } ops{d, m, ring, emptyc, fullh, H_ready, abort_flag, stb, pol, r0, nowait};
+            run_fields_warp(ops, nk, nb, L);
         }
     } else if (warp >= W) {
         // ---------------- fold warp of replica w ----------------
