@@ -19,6 +19,7 @@
 // N = 300007 with one replica (a launch per class) 30.8 -> 16, N = 20011 with four 24.9 -> 16.1.
 // Without the rings there is no pipeline to fill and drain in each class, and no launch gap.
 #include <algorithm>
+#include <type_traits>
 
 #include "../../include/sg.h"
 #include "sg_internal.cuh"
@@ -37,7 +38,13 @@ struct SweepShape {
 };
 
 constexpr int kSweepTables = 32;  // graphs whose thresholds are kept in shared memory
-constexpr int kSweepPlanes = 4;  // counter planes: slices up to width 15; wider ones count apart
+// Counter planes: slices up to width 15, and wider ones (degrees up to 63).  Both take their entries in
+// chunks: one entry at a time, each waiting for its slot and then its words, a class lasts as long as its
+// widest slice (us a sweep, one at a time -> chunks: N = 20000, degree 12, R = 2 55.8 -> 29.2, R = 4
+// 102 -> 37; N = 200000, degree 16, R = 2 82.7 -> 45.7; also N = 2^23, degree 4, R = 2 297 -> 282, where a few
+// slices of the first class are wider than 15).
+constexpr int kSweepPlanes = 4, kSweepWidePlanes = 6;
+static_assert(SG_VB_MAX_DEGREE < (1 << kSweepWidePlanes), "the counter holds every degree");
 
 __device__ __forceinline__ uint32_t ld_stream_u32(const uint32_t* p, uint64_t pol) {
     uint32_t v;
@@ -251,12 +258,13 @@ __global__ void __launch_bounds__(SweepShape<R, kChunk>::threads, 2)
                 nnm = load_meta(nn);
                 nnvi = load_vi(nn);
             };
-            if (left < (1u << kSweepPlanes)) {
-                uint64_t p[R][kSweepPlanes];
+            auto count = [&](auto planes) {
+                constexpr int P = decltype(planes)::value;
+                uint64_t p[R][P];
 #pragma unroll
                 for (int r = 0; r < R; ++r)
 #pragma unroll
-                    for (int b = 0; b < kSweepPlanes; ++b) p[r][b] = 0ull;
+                    for (int b = 0; b < P; ++b) p[r][b] = 0ull;
                 for (;;) {
                     SpinWords<R> g[kChunk];
                     uint64_t Jc[kChunk];
@@ -279,29 +287,16 @@ __global__ void __launch_bounds__(SweepShape<R, kChunk>::threads, 2)
                         uint64_t x[kChunk];
 #pragma unroll
                         for (int e = 0; e < kChunk; ++e) x[e] = si.v[r] ^ g[e].v[r] ^ Jc[e];
-                        bitslice_add4<kSweepPlanes>(p[r], x[0], x[1], x[2], x[3]);
-                        if constexpr (kChunk == 8) bitslice_add4<kSweepPlanes>(p[r], x[4], x[5], x[6], x[7]);
+                        bitslice_add4<P>(p[r], x[0], x[1], x[2], x[3]);
+                        if constexpr (kChunk == 8) bitslice_add4<P>(p[r], x[4], x[5], x[6], x[7]);
                     }
                     if (last) break;
                 }
 #pragma unroll
-                for (int r = 0; r < R; ++r) si.v[r] ^= at_least<kSweepPlanes>(p[r], kmin[r]);
-            } else {
-                uint64_t p[R][6];
-#pragma unroll
-                for (int r = 0; r < R; ++r)
-#pragma unroll
-                    for (int b = 0; b < 6; ++b) p[r][b] = 0ull;
-                for (uint32_t e = 0; e < left; ++e, idx += 32) {
-                    const uint64_t Je = __ldg(d.jb + idx);
-                    const SpinWords<R> sj = ld_spins<R>(d.S + (int64_t)__ldg(d.col + idx) * R, pol_keep);
-#pragma unroll
-                    for (int r = 0; r < R; ++r) bitslice_add<6>(p[r], si.v[r] ^ sj.v[r] ^ Je);
-                }
-#pragma unroll
-                for (int r = 0; r < R; ++r) si.v[r] ^= at_least<6>(p[r], kmin[r]);
-                advance();
-            }
+                for (int r = 0; r < R; ++r) si.v[r] ^= at_least<P>(p[r], kmin[r]);
+            };
+            if (left < (1u << kSweepPlanes)) count(std::integral_constant<int, kSweepPlanes>{});
+            else count(std::integral_constant<int, kSweepWidePlanes>{});
             // a warp's only slice comes next again: its words were read ahead of this update
             if (nx.slice == slice) nsi = si;
             if (vi != kInactive)

@@ -1,0 +1,79 @@
+"""Slices at the widths where the packed sweeps change their counting (chunks of 4 or 8 entries, four or
+six counter planes), every vertex of the same degree: one CTA, a cluster, grid-wide with at most one slice
+a warp and with several.  Spins equal the oracle's.  A slice of 16 entries takes as many rounds of gathers as one of 15
+and two more planes: its sweep may take half as long again, and no more."""
+import numpy as np
+import pytest
+
+import oracle
+import sg_inputs
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+TEMPS = [1.0, 0.6, 3.0, 0.0]
+
+
+@pytest.fixture(scope="module")
+def sg():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1906_11195_gb300 as m
+    return m
+
+
+def circulant(n, z):
+    """Vertex i of the left half is joined to the right half's i + a for z random offsets a."""
+    h = n // 2
+    a = np.random.default_rng(n + z).choice(h, z, replace=False)
+    i = np.arange(h)[:, None]
+    col = np.concatenate([h + np.sort((i + a) % h, axis=1), np.sort((i - a) % h, axis=1)])
+    src = np.repeat(np.arange(n), z)
+    lo, hi = np.minimum(src, col.ravel()), np.maximum(src, col.ravel())
+    eid = np.unique(lo * n + hi, return_inverse=True)[1]
+    return (np.arange(n + 1) * z).astype(np.int32), col.ravel().astype(np.int32), eid
+
+
+def instance(graph, z, R):
+    rp, col, eid = graph
+    jb = sg_inputs.vb_lane_couplings(eid, int(eid.max()) + 1, 3)
+    return dict(row_ptr=rp, col=col, jbits=jb, seed=(5 << 32) + z, temps=TEMPS[:R])
+
+
+@pytest.mark.parametrize("R", [1, 2, 4])
+@pytest.mark.parametrize("n,z", [(n, z) for n in (200, 3000, 30000) for z in (15, 16, 17, 20, 24, 25, 31, 32, 63)] +
+                         [(250_000, 17), (250_000, 25)])
+def test_spins(sg, n, z, R):
+    g = instance(circulant(n, z), z, R)
+    run = sg.VBRun([g], n_lanes=64, n_replicas=R)
+    run.sweep(1)
+    run.sweep(3)
+    run.synchronize()
+    spins = run.spins()[0]
+    run.close()
+    lanes = 64 if n <= 3000 else 3 if n < 100_000 else 1
+    mask = np.uint64((1 << lanes) - 1)
+    ref = oracle.vb_run(g["row_ptr"], g["col"], g["jbits"], lanes, g["temps"], g["seed"], 4, [], [])
+    assert np.array_equal(spins & mask, ref["spins"] & mask)
+
+
+def us_per_sweep(sg, n, z, R, sweeps=32):
+    run = sg.VBRun([instance(sg_inputs.random_regular_graph(n, z, 3, bipartite=True), z, R)], n_lanes=64, n_replicas=R)
+    run.sweep(sweeps)
+    a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+    times = []
+    for _ in range(7):
+        a.record()
+        run.sweep(sweeps)
+        b.record()
+        torch.cuda.synchronize()
+        times.append(a.elapsed_time(b) / sweeps * 1e3)
+    run.synchronize()
+    run.close()
+    return sorted(times)[3]
+
+
+@pytest.mark.parametrize("R", [1, 2, 4])
+@pytest.mark.parametrize("n", [30000, 200_000])
+def test_a_sweep_of_width_16_takes_about_as_long_as_one_of_15(sg, n, R):
+    assert us_per_sweep(sg, n, 16, R) <= 1.5 * us_per_sweep(sg, n, 15, R)
