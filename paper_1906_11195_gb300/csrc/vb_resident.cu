@@ -20,6 +20,8 @@
 //
 // The slices (32 vertices) of a class are dealt in turn to the CTAs of the cluster, and in a CTA to
 // its warps.
+#include <type_traits>
+
 #include "../../include/sg.h"
 #include "sg_internal.cuh"
 #include "vb_bits.cuh"
@@ -29,7 +31,11 @@ namespace sg {
 
 namespace {
 
-constexpr int kResPlanes = 4;  // counter planes: slices up to width 15; wider ones count apart
+// Counter planes: slices up to width 15, and wider ones (degrees up to 63).  Both take their entries in
+// chunks: one at a time a class lasts as long as its widest slice (us a sweep, one at a time -> chunks:
+// N = 3000, degree 16, R = 2 19.1 -> 14.4, R = 4 126 -> 38; degree 24, R = 2 114 -> 54).
+constexpr int kResPlanes = 4, kResWidePlanes = 6;
+static_assert(SG_VB_MAX_DEGREE < (1 << kResWidePlanes), "the counter holds every degree");
 
 __device__ __forceinline__ uint32_t cluster_rank() {
     uint32_t r;
@@ -233,7 +239,7 @@ __global__ void __launch_bounds__(kResThreads, 1)
                 const uint32_t i = ((l - first_of[c][rank]) << lc) + rank;  // the slice's place in its class
                 uint64_t* own = S + ((MODE == kResCopies ? c_before[c] + i : l) * 32 + lane) * R;
                 SpinWords<R> si = load_words<R>(own);
-                uint32_t e = base[l] + lane;
+                const uint32_t e = base[l] + lane;
                 const uint32_t end = base[l + 1];  // width = (end - base[l]) / 32
                 const uint32_t vi = vinfo[l * 32 + lane];
                 const uint8_t* k = kmins + ((size_t)(t & 1u) * rs.max_slices * 32 + l * 32 + lane) * R;
@@ -245,51 +251,55 @@ __global__ void __launch_bounds__(kResThreads, 1)
 #pragma unroll
                     for (int r = 0; r < R; ++r) kmin[r] = (int)((packed >> (8 * r)) & 255u);
                 }
-                if (end - base[l] <= 32u * ((1u << kResPlanes) - 1u)) {
-                    constexpr int CH = R == 4 ? 4 : 8;  // entries whose words are on their way at once
-                    uint64_t p[R][kResPlanes];
+                // count and flip replicas r0 .. r0 + RW - 1, the words of CH entries on their way at once
+                auto count = [&](auto planes, auto replicas, auto first, auto chunk) {
+                    constexpr int P = decltype(planes)::value, RW = decltype(replicas)::value;
+                    constexpr int r0 = decltype(first)::value, CH = decltype(chunk)::value;
+                    uint64_t p[RW][P];
 #pragma unroll
-                    for (int r = 0; r < R; ++r)
+                    for (int r = 0; r < RW; ++r)
 #pragma unroll
-                        for (int b = 0; b < kResPlanes; ++b) p[r][b] = 0ull;
-                    for (; e < end; e += 32 * CH) {
-                        SpinWords<R> w[CH];
+                        for (int b = 0; b < P; ++b) p[r][b] = 0ull;
+                    for (uint32_t i = e; i < end; i += 32 * CH) {
+                        SpinWords<RW> w[CH];
                         uint64_t Je[CH];
 #pragma unroll
                         for (int u = 0; u < CH; ++u) {
-                            w[u] = si;  // an absent entry counts nothing
+#pragma unroll
+                            for (int r = 0; r < RW; ++r) w[u].v[r] = si.v[r0 + r];  // an absent entry counts nothing
                             Je[u] = 0ull;
-                            if (e + 32 * u < end) {
-                                w[u] = gather_near<R, MODE>(nbr[e + 32 * u]);
-                                Je[u] = J[e + 32 * u];
+                            if (i + 32 * u < end) {
+                                w[u] = gather_near<RW, MODE>(nbr[i + 32 * u] + 8 * r0);
+                                Je[u] = J[i + 32 * u];
                             }
                         }
 #pragma unroll
                         for (int h = 0; h < CH; h += 4) {
-                            if (e + 32 * h >= end) break;  // warp-uniform
+                            if (i + 32 * h >= end) break;  // warp-uniform
 #pragma unroll
-                            for (int r = 0; r < R; ++r)
-                                bitslice_add4<kResPlanes>(p[r], si.v[r] ^ w[h].v[r] ^ Je[h],
-                                                          si.v[r] ^ w[h + 1].v[r] ^ Je[h + 1],
-                                                          si.v[r] ^ w[h + 2].v[r] ^ Je[h + 2],
-                                                          si.v[r] ^ w[h + 3].v[r] ^ Je[h + 3]);
+                            for (int r = 0; r < RW; ++r)
+                                bitslice_add4<P>(p[r], si.v[r0 + r] ^ w[h].v[r] ^ Je[h],
+                                                 si.v[r0 + r] ^ w[h + 1].v[r] ^ Je[h + 1],
+                                                 si.v[r0 + r] ^ w[h + 2].v[r] ^ Je[h + 2],
+                                                 si.v[r0 + r] ^ w[h + 3].v[r] ^ Je[h + 3]);
                         }
                     }
 #pragma unroll
-                    for (int r = 0; r < R; ++r) si.v[r] ^= at_least<kResPlanes>(p[r], kmin[r]);
+                    for (int r = 0; r < RW; ++r) si.v[r0 + r] ^= at_least<P>(p[r], kmin[r0 + r]);
+                };
+                using std::integral_constant;
+                if (end - base[l] <= 32u * ((1u << kResPlanes) - 1u)) {
+                    count(integral_constant<int, kResPlanes>{}, integral_constant<int, R>{},
+                          integral_constant<int, 0>{}, integral_constant<int, R == 4 ? 4 : 8>{});
                 } else {
-                    uint64_t p[R][6];
-#pragma unroll
-                    for (int r = 0; r < R; ++r)
-#pragma unroll
-                        for (int b = 0; b < 6; ++b) p[r][b] = 0ull;
-                    for (; e < end; e += 32) {
-                        const SpinWords<R> w = gather_near<R, MODE>(nbr[e]);
-#pragma unroll
-                        for (int r = 0; r < R; ++r) bitslice_add<6>(p[r], si.v[r] ^ w.v[r] ^ J[e]);
-                    }
-#pragma unroll
-                    for (int r = 0; r < R; ++r) si.v[r] ^= at_least<6>(p[r], kmin[r]);
+                    // wider: six planes, and of four replicas two at a time (all four would need more
+                    // than the 96 registers of 18 warps)
+                    constexpr int RW = R == 1 ? 1 : 2;
+                    count(integral_constant<int, kResWidePlanes>{}, integral_constant<int, RW>{},
+                          integral_constant<int, 0>{}, integral_constant<int, 8>{});
+                    if constexpr (R == 4)
+                        count(integral_constant<int, kResWidePlanes>{}, integral_constant<int, RW>{},
+                              integral_constant<int, 2>{}, integral_constant<int, 8>{});
                 }
                 if (vi != kInactive) {
 #pragma unroll

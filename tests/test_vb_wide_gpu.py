@@ -58,7 +58,7 @@ def test_spins(sg, n, z, R):
 
 
 def us_per_sweep(sg, n, z, R, sweeps=32):
-    run = sg.VBRun([instance(sg_inputs.random_regular_graph(n, z, 3, bipartite=True), z, R)], n_lanes=64, n_replicas=R)
+    run = sg.VBRun([instance(circulant(n, z) if n < 1000 else sg_inputs.random_regular_graph(n, z, 3, bipartite=True), z, R)], n_lanes=64, n_replicas=R)
     run.sweep(sweeps)
     a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
     times = []
@@ -74,6 +74,13 @@ def us_per_sweep(sg, n, z, R, sweeps=32):
 
 
 @pytest.mark.parametrize("R", [1, 2, 4])
-@pytest.mark.parametrize("n", [30000, 200_000])
+@pytest.mark.parametrize("n", [200, 3000, 8000, 30000, 200_000])
 def test_a_sweep_of_width_16_takes_about_as_long_as_one_of_15(sg, n, R):
     assert us_per_sweep(sg, n, 16, R) <= 1.5 * us_per_sweep(sg, n, 15, R)
+
+
+@pytest.mark.parametrize("R", [1, 2, 4])
+@pytest.mark.parametrize("n", [200, 3000, 8000])
+def test_time_grows_no_faster_than_the_entries(sg, n, R):
+    """By a quarter more at most, for the two more planes of the wide slices."""
+    assert us_per_sweep(sg, n, 31, R) <= 5 / 4 * 31 / 15 * us_per_sweep(sg, n, 15, R)
