@@ -276,8 +276,9 @@ public:
         check_cuda(cudaStreamSynchronize(st), "attach");
     }
 
-    // The plan with 2^lc CTAs for every graph; false: some graph does not fit.
-    bool resident_layout(uint32_t lc, bool copies, VbResident& rs) const {
+    // The plan with 2^lc CTAs for every graph, and the entries of the largest graph; false: some graph does
+    // not fit.
+    bool resident_layout(uint32_t lc, bool copies, VbResident& rs, int64_t& graph_entries) const {
         const int nc = pk_.n_colours;
         const uint32_t C = 1u << lc;
         rs = rs_;
@@ -287,8 +288,9 @@ public:
         rs.graph_slices = 0;
         rs.max_slices = 0;
         rs.max_entries = 0;
+        graph_entries = 0;
         for (int b = 0; b < n_inst; ++b) {
-            int64_t ns[kResMaxCluster] = {}, ne[kResMaxCluster] = {}, all = 0;
+            int64_t ns[kResMaxCluster] = {}, ne[kResMaxCluster] = {}, all = 0, entries = 0;
             for (int c = 0; c < nc; ++c) {
                 const uint32_t lo = graph_class_slice_[(size_t)c * n_inst + b],
                                hi = graph_class_slice_[(size_t)c * n_inst + b + 1];
@@ -303,13 +305,38 @@ public:
             for (uint32_t k = 0; k < C; ++k) {
                 rs.max_slices = std::max(rs.max_slices, (int)ns[k]);
                 rs.max_entries = std::max(rs.max_entries, (uint32_t)ne[k]);
+                entries += ne[k];
             }
+            graph_entries = std::max(graph_entries, entries);
             rs.graph_slices = std::max(rs.graph_slices, (int)all);
             if (vb_resident_smem(R, copies ? rs.graph_slices : rs.max_slices, rs.max_slices,
                                  rs.max_entries) > (size_t)kResMaxSmem)
                 return false;
         }
         return vb_resident_clusters(R, rs) >= n_inst;
+    }
+
+    // What a class takes in a cluster, and grid-wide (us, the average over the classes), for one, two and
+    // four replicas.  Fitted to bipartite graphs of degree 3 to 6 and Poissonian ones of mean degree 2 to 16,
+    // N = 1000 .. 48000, alone and in batches of up to 100; within 15 %.
+    // With copies of all words a CTA sends each slice that it updates to the others; without, it gathers
+    // its slices' entries, a row of 32 at a time, from them.  Examples (us a sweep, one replica where not
+    // said, cluster against grid): bipartite N = 8192 3.6, 4.0; 16384 5.7, 4.1; 32768 13.5, 4.2; two replicas
+    // 4096 3.0, 4.5; 16384 7.8, 4.6; four replicas 4096 4.8, 4.9; 8192 8.2, 4.9; Poissonian of degree 4,
+    // N = 16384 8.1, 10.9; 24000 14.5, 11.6; nine bipartite graphs of 9000, two replicas, 6.0, 6.8.
+    double cluster_us(const VbResident& rs, int64_t graph_entries, int more) const {
+        static const double kCopies[3][3] = {{0.8, 0.03, 0.0065}, {0.75, 0.04, 0.0125}, {1.5, 0.06, 0.04}};
+        static const double kGather[3][3] = {{0.95, 0.045, 0.15}, {0.85, 0.047, 0.25}, {0.9, 0.096, 0.6}};
+        const int q = R == 4 ? 2 : R - 1;
+        const double slices = (double)rs.max_slices / pk_.n_colours;
+        const double rows = (double)graph_entries / rs.cluster / 32 / pk_.n_colours;
+        if (rs.copies) return kCopies[q][0] + slices * (kCopies[q][1] + kCopies[q][2] * (rs.cluster - 1));
+        return kGather[q][0] + rows * kGather[q][1] + more * kGather[q][2];
+    }
+    double grid_us(int more) const {
+        static const double kGridWide[3][3] = {{2.0, 0.00055, 0.15}, {2.2, 0.0007, 0.3}, {2.4, 0.00105, 0.33}};
+        const int q = R == 4 ? 2 : R - 1;
+        return kGridWide[q][0] + kGridWide[q][1] * pk_.n_slices / pk_.n_colours + more * kGridWide[q][2];
     }
 
     // Which graphs run in shared memory, and how (R = 2, Poissonian of degree 4, us a sweep).
@@ -320,12 +347,9 @@ public:
     // one replica, N = 18000 8.3, 11.4).  Each update goes to all CTAs, so four replicas do not gain
     // from 16 (N = 4500 13.6, without copies 10.9), nor does a graph of degree 4, whose words
     // arrive in one round (bipartite N = 4096: 16 CTAs without copies 2.9, 8 with copies 3.2).
-    // Without copies up to 104 KB of words gathered by a CTA in a sweep: gathers from other CTAs' shared
-    // memory take about 4 cycles for each 16 bytes, and there the grid-wide form draws level
-    // (N = 40000, 170 KB: 22.9 against 16.9; N = 20011, four replicas, 175 KB: 22.7 against 18.3).
+    // A cluster only where it is estimated to take no longer than the grid-wide form.
     // A batch takes the first of these for which the GPU holds all its clusters at once.
     bool plan_resident() {
-        constexpr int64_t kMaxGatherBytes = 104 * 1024;
         if (pk_.n_colours < 1) return false;
         int widest = 0;  // slices of the largest class of one graph
         for (size_t i = 0; i + 1 < graph_class_slice_.size(); ++i)
@@ -333,10 +357,12 @@ public:
         uint32_t width = 0;  // entries of the widest slice
         for (size_t i = 0; i + 1 < h_slice_base_.size(); ++i)
             width = std::max(width, (h_slice_base_[i + 1] - h_slice_base_[i]) / 32);
+        const int more = width > 8 ? (int)(width - 1) / 8 : 0;
         VbResident rs;
+        int64_t entries = 0;
         auto take = [&](uint32_t lc, bool copies) {
-            if (!resident_layout(lc, copies, rs)) return false;
-            if (lc > 0 && !copies && (int64_t)rs.max_entries * R * 8 > kMaxGatherBytes) return false;
+            if (!resident_layout(lc, copies, rs, entries)) return false;
+            if (lc > 0 && cluster_us(rs, entries, more) > grid_us(more)) return false;
             rs_ = rs;
             return true;
         };

@@ -1,0 +1,67 @@
+"""Which form a Viana-Bray handle's sweeps take: a sweep of a graph takes no longer than one of a graph of
+the same kind and twice its size, by a quarter at most, whichever of them run in shared memory; spins on
+both sides of the line between a cluster and the grid equal the oracle's."""
+import numpy as np
+import pytest
+
+import oracle
+import sg_inputs
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+TEMPS = [1.0, 0.6, 3.0, 0.0]
+
+
+@pytest.fixture(scope="module")
+def sg():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1906_11195_gb300 as m
+    return m
+
+
+def instance(n, z, R, k=0):
+    rp, col, eid = sg_inputs.random_regular_graph(n, z, 3 + k, bipartite=True)
+    jb = sg_inputs.vb_lane_couplings(eid, n * z // 2, 3 + k)
+    return dict(row_ptr=rp, col=col, jbits=jb, seed=(5 << 32) + k, temps=TEMPS[:R])
+
+
+def us(call, n=1, runs=9):
+    a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+    times = []
+    for _ in range(runs):
+        a.record()
+        call()
+        b.record()
+        torch.cuda.synchronize()
+        times.append(a.elapsed_time(b) / n * 1e3)
+    return sorted(times)[runs // 2]
+
+
+@pytest.mark.parametrize("R", [1, 2, 4])
+def test_a_sweep_takes_no_longer_than_one_of_twice_the_vertices(sg, R):
+    t = {}
+    for n in (4096, 8192, 16384, 32768, 65536):
+        run = sg.VBRun([instance(n, 4, R)], n_lanes=64, n_replicas=R)
+        run.sweep(64)
+        t[n] = us(lambda: run.sweep(64), 64)
+        run.synchronize()
+        run.close()
+    for n in list(t)[:-1]:
+        assert t[n] <= 1.25 * t[2 * n], t
+
+
+@pytest.mark.parametrize("R", [1, 2, 4])
+@pytest.mark.parametrize("n,z,count", [(2048, 6, 1), (8192, 4, 1), (12000, 3, 1), (24000, 4, 1), (9000, 4, 4)])
+def test_spins(sg, n, z, count, R):
+    graphs = [instance(n, z, R, k) for k in range(count)]
+    run = sg.VBRun(graphs, n_lanes=64, n_replicas=R)
+    for m in (3, 1, 2):
+        run.sweep(m)
+    run.synchronize()
+    spins = run.spins()
+    run.close()
+    for g, s in zip(graphs, spins):
+        ref = oracle.vb_run(g["row_ptr"], g["col"], g["jbits"], 5, g["temps"], g["seed"], 6, [], [])
+        assert np.array_equal(s & np.uint64(31), ref["spins"] & np.uint64(31))
