@@ -185,6 +185,7 @@ struct VbPackedDev {
     int32_t R;
     int32_t n_colours;
     int32_t n_graphs;
+    uint32_t max_width;          // entries of the widest slice
     const uint32_t* class_slice; // [n_colours+1] first slice of each colour class
     bool stream_first;           // the graph does not fit L2 beside the spins: its lines leave first
     uint64_t stage_wait_ns;      // bound of one wait at the sweeps' grid barrier

@@ -354,9 +354,8 @@ public:
         int widest = 0;  // slices of the largest class of one graph
         for (size_t i = 0; i + 1 < graph_class_slice_.size(); ++i)
             widest = std::max(widest, (int)(graph_class_slice_[i + 1] - graph_class_slice_[i]));
-        uint32_t width = 0;  // entries of the widest slice
-        for (size_t i = 0; i + 1 < h_slice_base_.size(); ++i)
-            width = std::max(width, (h_slice_base_[i + 1] - h_slice_base_[i]) / 32);
+        const uint32_t width = pk_.max_width;
+        rs_.wide = width > 15;
         const int more = width > 8 ? (int)(width - 1) / 8 : 0;
         VbResident rs;
         int64_t entries = 0;
@@ -668,6 +667,7 @@ private:
             pk_.n_slices = (int32_t)(n_slots_ / 32);
             pk_.R = R;
             pk_.n_graphs = n_inst;
+            pk_.max_width = max_width_;
             pk_.n_colours = (int32_t)colour_slice_.size() - 1;
             // SG_TEST_STAGE_WAIT_NS shortens the colour kernel's pipeline waits: a test of the
             // timeout path (the kernel gives up, flags SG_ETIMEOUT and exits cleanly)
@@ -801,6 +801,7 @@ private:
         });
         int64_t entries = 0;
         for (int64_t s = 0; s < n_slices; ++s) {
+            max_width_ = std::max(max_width_, (uint32_t)width_of[s]);
             h_slice_base_[s] = (uint32_t)entries;
             entries += 32 * (int64_t)width_of[s];
             if (entries >= (int64_t(1) << 32)) fail(SG_EINVAL, "too many graph entries for one batch");
@@ -873,6 +874,7 @@ private:
     enum Form { kGrid, kResident };
     Form form_ = kGrid;         // vb_sweep.cu or vb_resident.cu, chosen at attach
     int max_class_slices_ = 0;  // slices of the largest class
+    uint32_t max_width_ = 0;    // entries of the widest slice
     VbResident rs_{};
     std::vector<uint32_t> graph_class_slice_;  // first slice of every (class, graph)
     int Lc_ = 64;

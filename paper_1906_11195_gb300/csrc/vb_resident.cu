@@ -20,8 +20,6 @@
 //
 // The slices (32 vertices) of a class are dealt in turn to the CTAs of the cluster, and in a CTA to
 // its warps.
-#include <type_traits>
-
 #include "../../include/sg.h"
 #include "sg_internal.cuh"
 #include "vb_bits.cuh"
@@ -33,7 +31,9 @@ namespace {
 
 // Counter planes: slices up to width 15, and wider ones (degrees up to 63).  Both take their entries in
 // chunks: one at a time a class lasts as long as its widest slice (us a sweep, one at a time -> chunks:
-// N = 3000, degree 16, R = 2 19.1 -> 14.4, R = 4 126 -> 38; degree 24, R = 2 114 -> 54).
+// N = 3000, degree 16, R = 2 19.1 -> 14.4, R = 4 126 -> 38; degree 24, R = 2 114 -> 54).  Graphs without wide
+// slices run kernels without their counting, whose registers would slow the others down (R = 4, N = 1500
+// 8.2 us a sweep, 8.6 with it).
 constexpr int kResPlanes = 4, kResWidePlanes = 6;
 static_assert(SG_VB_MAX_DEGREE < (1 << kResWidePlanes), "the counter holds every degree");
 
@@ -90,7 +90,7 @@ __device__ __forceinline__ void class_barrier_wait() {
 
 }  // namespace
 
-template <int R, int MODE>
+template <int R, int MODE, bool WIDE>
 __global__ void __launch_bounds__(kResThreads, 1)
     k_vb_resident(VbPackedDev d, VbResident rs, uint32_t t0, uint32_t n_sweeps) {
     extern __shared__ __align__(128) uint8_t smem[];
@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(kResThreads, 1)
                 const uint32_t i = ((l - first_of[c][rank]) << lc) + rank;  // the slice's place in its class
                 uint64_t* own = S + ((MODE == kResCopies ? c_before[c] + i : l) * 32 + lane) * R;
                 SpinWords<R> si = load_words<R>(own);
-                const uint32_t e = base[l] + lane;
+                uint32_t e = base[l] + lane;
                 const uint32_t end = base[l + 1];  // width = (end - base[l]) / 32
                 const uint32_t vi = vinfo[l * 32 + lane];
                 const uint8_t* k = kmins + ((size_t)(t & 1u) * rs.max_slices * 32 + l * 32 + lane) * R;
@@ -251,55 +251,93 @@ __global__ void __launch_bounds__(kResThreads, 1)
 #pragma unroll
                     for (int r = 0; r < R; ++r) kmin[r] = (int)((packed >> (8 * r)) & 255u);
                 }
-                // count and flip replicas r0 .. r0 + RW - 1, the words of CH entries on their way at once
-                auto count = [&](auto planes, auto replicas, auto first, auto chunk) {
-                    constexpr int P = decltype(planes)::value, RW = decltype(replicas)::value;
-                    constexpr int r0 = decltype(first)::value, CH = decltype(chunk)::value;
-                    uint64_t p[RW][P];
+                // (in one CTA with four replicas the compiler orders the loads of narrow slices better beside
+                // a plain loop for wide ones, which no graph of such a launch has: N = 300 4.75 us a sweep,
+                // without 5.0; N = 1000 7.43, 7.66)
+                constexpr bool kPlainWide = !WIDE && R == 4 && MODE == kResSolo;
+                if ((!WIDE && !kPlainWide) || end - base[l] <= 32u * ((1u << kResPlanes) - 1u)) {
+                    constexpr int CH = R == 4 ? 4 : 8;  // entries whose words are on their way at once
+                    uint64_t p[R][kResPlanes];
 #pragma unroll
-                    for (int r = 0; r < RW; ++r)
+                    for (int r = 0; r < R; ++r)
 #pragma unroll
-                        for (int b = 0; b < P; ++b) p[r][b] = 0ull;
-                    for (uint32_t i = e; i < end; i += 32 * CH) {
-                        SpinWords<RW> w[CH];
+                        for (int b = 0; b < kResPlanes; ++b) p[r][b] = 0ull;
+                    for (; e < end; e += 32 * CH) {
+                        SpinWords<R> w[CH];
                         uint64_t Je[CH];
 #pragma unroll
                         for (int u = 0; u < CH; ++u) {
-#pragma unroll
-                            for (int r = 0; r < RW; ++r) w[u].v[r] = si.v[r0 + r];  // an absent entry counts nothing
+                            w[u] = si;  // an absent entry counts nothing
                             Je[u] = 0ull;
-                            if (i + 32 * u < end) {
-                                w[u] = gather_near<RW, MODE>(nbr[i + 32 * u] + 8 * r0);
-                                Je[u] = J[i + 32 * u];
+                            if (e + 32 * u < end) {
+                                w[u] = gather_near<R, MODE>(nbr[e + 32 * u]);
+                                Je[u] = J[e + 32 * u];
                             }
                         }
 #pragma unroll
                         for (int h = 0; h < CH; h += 4) {
-                            if (i + 32 * h >= end) break;  // warp-uniform
+                            if (e + 32 * h >= end) break;  // warp-uniform
 #pragma unroll
-                            for (int r = 0; r < RW; ++r)
-                                bitslice_add4<P>(p[r], si.v[r0 + r] ^ w[h].v[r] ^ Je[h],
-                                                 si.v[r0 + r] ^ w[h + 1].v[r] ^ Je[h + 1],
-                                                 si.v[r0 + r] ^ w[h + 2].v[r] ^ Je[h + 2],
-                                                 si.v[r0 + r] ^ w[h + 3].v[r] ^ Je[h + 3]);
+                            for (int r = 0; r < R; ++r)
+                                bitslice_add4<kResPlanes>(p[r], si.v[r] ^ w[h].v[r] ^ Je[h],
+                                                          si.v[r] ^ w[h + 1].v[r] ^ Je[h + 1],
+                                                          si.v[r] ^ w[h + 2].v[r] ^ Je[h + 2],
+                                                          si.v[r] ^ w[h + 3].v[r] ^ Je[h + 3]);
                         }
                     }
 #pragma unroll
-                    for (int r = 0; r < RW; ++r) si.v[r0 + r] ^= at_least<P>(p[r], kmin[r0 + r]);
-                };
-                using std::integral_constant;
-                if (end - base[l] <= 32u * ((1u << kResPlanes) - 1u)) {
-                    count(integral_constant<int, kResPlanes>{}, integral_constant<int, R>{},
-                          integral_constant<int, 0>{}, integral_constant<int, R == 4 ? 4 : 8>{});
-                } else {
-                    // wider: six planes, and of four replicas two at a time (all four would need more
-                    // than the 96 registers of 18 warps)
-                    constexpr int RW = R == 1 ? 1 : 2;
-                    count(integral_constant<int, kResWidePlanes>{}, integral_constant<int, RW>{},
-                          integral_constant<int, 0>{}, integral_constant<int, 8>{});
-                    if constexpr (R == 4)
-                        count(integral_constant<int, kResWidePlanes>{}, integral_constant<int, RW>{},
-                              integral_constant<int, 2>{}, integral_constant<int, 8>{});
+                    for (int r = 0; r < R; ++r) si.v[r] ^= at_least<kResPlanes>(p[r], kmin[r]);
+                } else if constexpr (WIDE) {
+                    // six planes, and of four replicas two at a time (all four would need more than the 96
+                    // registers of 18 warps)
+                    constexpr int RW = R == 1 ? 1 : 2, CH = 8;
+#pragma unroll
+                    for (int r0 = 0; r0 < R; r0 += RW) {
+                        uint64_t p[RW][kResWidePlanes];
+#pragma unroll
+                        for (int r = 0; r < RW; ++r)
+#pragma unroll
+                            for (int b = 0; b < kResWidePlanes; ++b) p[r][b] = 0ull;
+                        for (uint32_t i = e; i < end; i += 32 * CH) {
+                            SpinWords<RW> w[CH];
+                            uint64_t Je[CH];
+#pragma unroll
+                            for (int u = 0; u < CH; ++u) {
+#pragma unroll
+                                for (int r = 0; r < RW; ++r) w[u].v[r] = si.v[r0 + r];
+                                Je[u] = 0ull;
+                                if (i + 32 * u < end) {
+                                    w[u] = gather_near<RW, MODE>(nbr[i + 32 * u] + 8 * r0);
+                                    Je[u] = J[i + 32 * u];
+                                }
+                            }
+#pragma unroll
+                            for (int h = 0; h < CH; h += 4) {
+                                if (i + 32 * h >= end) break;  // warp-uniform
+#pragma unroll
+                                for (int r = 0; r < RW; ++r)
+                                    bitslice_add4<kResWidePlanes>(p[r], si.v[r0 + r] ^ w[h].v[r] ^ Je[h],
+                                                                  si.v[r0 + r] ^ w[h + 1].v[r] ^ Je[h + 1],
+                                                                  si.v[r0 + r] ^ w[h + 2].v[r] ^ Je[h + 2],
+                                                                  si.v[r0 + r] ^ w[h + 3].v[r] ^ Je[h + 3]);
+                            }
+                        }
+#pragma unroll
+                        for (int r = 0; r < RW; ++r) si.v[r0 + r] ^= at_least<kResWidePlanes>(p[r], kmin[r0 + r]);
+                    }
+                } else if constexpr (kPlainWide) {
+                    uint64_t p[R][kResWidePlanes];
+#pragma unroll
+                    for (int r = 0; r < R; ++r)
+#pragma unroll
+                        for (int b = 0; b < kResWidePlanes; ++b) p[r][b] = 0ull;
+                    for (; e < end; e += 32) {
+                        const SpinWords<R> w = gather_near<R, MODE>(nbr[e]);
+#pragma unroll
+                        for (int r = 0; r < R; ++r) bitslice_add<kResWidePlanes>(p[r], si.v[r] ^ w.v[r] ^ J[e]);
+                    }
+#pragma unroll
+                    for (int r = 0; r < R; ++r) si.v[r] ^= at_least<kResWidePlanes>(p[r], kmin[r]);
                 }
                 if (vi != kInactive) {
 #pragma unroll
@@ -331,10 +369,10 @@ size_t vb_resident_smem(int R, int word_slices, int max_slices, int64_t max_entr
            ((size_t)max_slices + 1) * 4 + (size_t)max_slices * 64 * R;
 }
 
-template <int R, int MODE>
+template <int R, int MODE, bool WIDE>
 static cudaError_t resident_config(const VbResident& rs, int n_graphs, cudaLaunchConfig_t& cfg,
                                    cudaLaunchAttribute* attr) {
-    auto kern = k_vb_resident<R, MODE>;
+    auto kern = k_vb_resident<R, MODE, WIDE>;
     const size_t smem = vb_resident_smem(R, rs.copies ? rs.graph_slices : rs.max_slices, rs.max_slices, rs.max_entries);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kResMaxSmem);
     if (e != cudaSuccess) return e;
@@ -355,18 +393,18 @@ static cudaError_t resident_config(const VbResident& rs, int n_graphs, cudaLaunc
     return cudaSuccess;
 }
 
-template <int R, int MODE>
+template <int R, int MODE, bool WIDE>
 static int resident_clusters(const VbResident& rs) {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
     int n = 0;
-    if (resident_config<R, MODE>(rs, 1, cfg, attr) != cudaSuccess) {
+    if (resident_config<R, MODE, WIDE>(rs, 1, cfg, attr) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
     if constexpr (MODE == kResSolo) {
         int dev = 0, sms = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_vb_resident<R, MODE>, kResThreads,
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_vb_resident<R, MODE, WIDE>, kResThreads,
                                                           cfg.dynamicSmemBytes) != cudaSuccess ||
             cudaGetDevice(&dev) != cudaSuccess ||
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
@@ -375,56 +413,59 @@ static int resident_clusters(const VbResident& rs) {
         }
         return n * sms;
     }
-    if (cudaOccupancyMaxActiveClusters(&n, k_vb_resident<R, MODE>, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, k_vb_resident<R, MODE, WIDE>, &cfg) != cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
     return n;
 }
 
-template <int R>
+template <int R, bool WIDE>
 static int resident_clusters_mode(const VbResident& rs) {
-    return rs.cluster == 1 ? resident_clusters<R, kResSolo>(rs)
-           : rs.copies ? resident_clusters<R, kResCopies>(rs)
-                               : resident_clusters<R, kResCluster>(rs);
+    return rs.cluster == 1 ? resident_clusters<R, kResSolo, WIDE>(rs)
+           : rs.copies ? resident_clusters<R, kResCopies, WIDE>(rs)
+                               : resident_clusters<R, kResCluster, WIDE>(rs);
 }
 
 int vb_resident_clusters(int R, const VbResident& rs) {
     if (vb_resident_smem(R, rs.copies ? rs.graph_slices : rs.max_slices, rs.max_slices, rs.max_entries) > (size_t)kResMaxSmem) return 0;
     switch (R) {
-        case 1: return resident_clusters_mode<1>(rs);
-        case 2: return resident_clusters_mode<2>(rs);
-        case 4: return resident_clusters_mode<4>(rs);
+        case 1: return rs.wide ? resident_clusters_mode<1, true>(rs) : resident_clusters_mode<1, false>(rs);
+        case 2: return rs.wide ? resident_clusters_mode<2, true>(rs) : resident_clusters_mode<2, false>(rs);
+        case 4: return rs.wide ? resident_clusters_mode<4, true>(rs) : resident_clusters_mode<4, false>(rs);
         default: return 0;
     }
 }
 
-template <int R, int MODE>
+template <int R, int MODE, bool WIDE>
 static int resident_launch(const VbPackedDev& d, const VbResident& rs, uint32_t t0,
                            int n_sweeps, cudaStream_t st) {
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute attr[1];
-    if (resident_config<R, MODE>(rs, d.n_graphs, cfg, attr) != cudaSuccess) return -1;
+    if (resident_config<R, MODE, WIDE>(rs, d.n_graphs, cfg, attr) != cudaSuccess) return -1;
     cfg.stream = st;
-    return cudaLaunchKernelEx(&cfg, k_vb_resident<R, MODE>, d, rs, t0, (uint32_t)n_sweeps) ==
+    return cudaLaunchKernelEx(&cfg, k_vb_resident<R, MODE, WIDE>, d, rs, t0, (uint32_t)n_sweeps) ==
                    cudaSuccess ? 1 : -1;
 }
 
-template <int R>
+template <int R, bool WIDE>
 static int resident_launch_mode(const VbPackedDev& d, const VbResident& rs, uint32_t t0,
                                 int n_sweeps, cudaStream_t st) {
-    return rs.cluster == 1 ? resident_launch<R, kResSolo>(d, rs, t0, n_sweeps, st)
-           : rs.copies ? resident_launch<R, kResCopies>(d, rs, t0, n_sweeps, st)
-                               : resident_launch<R, kResCluster>(d, rs, t0, n_sweeps, st);
+    return rs.cluster == 1 ? resident_launch<R, kResSolo, WIDE>(d, rs, t0, n_sweeps, st)
+           : rs.copies ? resident_launch<R, kResCopies, WIDE>(d, rs, t0, n_sweeps, st)
+                               : resident_launch<R, kResCluster, WIDE>(d, rs, t0, n_sweeps, st);
 }
 
 int vb_resident_sweeps(const VbPackedDev& d, const VbResident& rs, uint32_t t0,
                        int n_sweeps, cudaStream_t st) {
     if (n_sweeps <= 0) return 0;
     switch (d.R) {
-        case 1: return resident_launch_mode<1>(d, rs, t0, n_sweeps, st);
-        case 2: return resident_launch_mode<2>(d, rs, t0, n_sweeps, st);
-        case 4: return resident_launch_mode<4>(d, rs, t0, n_sweeps, st);
+        case 1: return rs.wide ? resident_launch_mode<1, true>(d, rs, t0, n_sweeps, st)
+                               : resident_launch_mode<1, false>(d, rs, t0, n_sweeps, st);
+        case 2: return rs.wide ? resident_launch_mode<2, true>(d, rs, t0, n_sweeps, st)
+                               : resident_launch_mode<2, false>(d, rs, t0, n_sweeps, st);
+        case 4: return rs.wide ? resident_launch_mode<4, true>(d, rs, t0, n_sweeps, st)
+                               : resident_launch_mode<4, false>(d, rs, t0, n_sweeps, st);
         default: return -1;
     }
 }

@@ -21,6 +21,7 @@ struct VbResident {
     const uint32_t* graph_class_slice;  // [n_colours n_graphs + 1] first slice of each (class, graph)
     uint32_t cluster, log_cluster;
     bool copies;
+    bool wide;                          // some slice has more than 15 entries (vb_resident.cu: kResPlanes)
     int graph_slices;                   // slices of the largest graph
     int max_slices;                     // slices and entries of the fullest CTA
     uint32_t max_entries;

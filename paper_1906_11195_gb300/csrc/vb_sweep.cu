@@ -42,7 +42,8 @@ constexpr int kSweepTables = 32;  // graphs whose thresholds are kept in shared 
 // chunks: one entry at a time, each waiting for its slot and then its words, a class lasts as long as its
 // widest slice (us a sweep, one at a time -> chunks: N = 20000, degree 12, R = 2 55.8 -> 29.2, R = 4
 // 102 -> 37; N = 200000, degree 16, R = 2 82.7 -> 45.7; also N = 2^23, degree 4, R = 2 297 -> 282, where a few
-// slices of the first class are wider than 15).
+// slices of the first class are wider than 15).  Graphs without wide slices run kernels without their
+// counting, whose registers would slow the others down (N = 30000, R = 2 13.6 us a sweep, 13.9 with it).
 constexpr int kSweepPlanes = 4, kSweepWidePlanes = 6;
 static_assert(SG_VB_MAX_DEGREE < (1 << kSweepWidePlanes), "the counter holds every degree");
 
@@ -109,7 +110,7 @@ struct Cursor {
 
 }  // namespace
 
-template <int R, int kChunk>
+template <int R, int kChunk, bool kWide>
 __global__ void __launch_bounds__(SweepShape<R, kChunk>::threads, 2)
     k_vb_sweeps(VbPackedDev d, uint32_t t0, uint32_t n_sweeps) {
     __shared__ uint32_t cs[kVbMaxColours + 1];  // first slice of each class
@@ -295,8 +296,8 @@ __global__ void __launch_bounds__(SweepShape<R, kChunk>::threads, 2)
 #pragma unroll
                 for (int r = 0; r < R; ++r) si.v[r] ^= at_least<P>(p[r], kmin[r]);
             };
-            if (left < (1u << kSweepPlanes)) count(std::integral_constant<int, kSweepPlanes>{});
-            else count(std::integral_constant<int, kSweepWidePlanes>{});
+            if (!kWide || left < (1u << kSweepPlanes)) count(std::integral_constant<int, kSweepPlanes>{});
+            else if constexpr (kWide) count(std::integral_constant<int, kSweepWidePlanes>{});
             // a warp's only slice comes next again: its words were read ahead of this update
             if (nx.slice == slice) nsi = si;
             if (vi != kInactive)
@@ -330,11 +331,11 @@ __global__ void __launch_bounds__(SweepShape<R, kChunk>::threads, 2)
 template <int R, int CH>
 static int sweep_warps(int sms) { return SweepShape<R, CH>::threads / 32 * 2 * sms; }
 
-template <int R, int CH>
+template <int R, int CH, bool kWide>
 static int launch_sweeps(const VbPackedDev& d, int max_class_slices, int sms, uint32_t t0,
                          int n_sweeps, cudaStream_t st) {
     constexpr int threads = SweepShape<R, CH>::threads, warps = threads / 32;
-    auto kern = k_vb_sweeps<R, CH>;
+    auto kern = k_vb_sweeps<R, CH, kWide>;
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, 0) != cudaSuccess ||
         per_sm < 1)
@@ -363,24 +364,28 @@ static int launch_sweeps(const VbPackedDev& d, int max_class_slices, int sms, ui
 // N = 65536: 15.6 us a sweep, 16.6 with chunks of 4; R = 4, N = 60000: 23.3, 27.1).  Beyond that the
 // registers are better spent on more warps (R = 2, bipartite N = 2^18: 10.3 us with chunks of 4,
 // 11.9 with 8; Poissonian N = 2^22: 128, 145; R = 4, N = 10^6: 80, 90).
-template <int R>
+template <int R, bool kWide>
 static int launch_r(const VbPackedDev& d, int max_class_slices, uint32_t t0, int n_sweeps, cudaStream_t st) {
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
         return -1;
     if (max_class_slices <= sweep_warps<R, 8>(sms))
-        return launch_sweeps<R, 8>(d, max_class_slices, sms, t0, n_sweeps, st);
-    return launch_sweeps<R, 4>(d, max_class_slices, sms, t0, n_sweeps, st);
+        return launch_sweeps<R, 8, kWide>(d, max_class_slices, sms, t0, n_sweeps, st);
+    return launch_sweeps<R, 4, kWide>(d, max_class_slices, sms, t0, n_sweeps, st);
 }
 
 int vb_packed_sweeps(const VbPackedDev& d, int max_class_slices, uint32_t t0, int n_sweeps,
                      cudaStream_t st) {
     if (n_sweeps <= 0 || d.n_colours <= 0) return 0;
+    const bool wide = d.max_width >= (1u << kSweepPlanes);
     switch (d.R) {
-        case 1: return launch_r<1>(d, max_class_slices, t0, n_sweeps, st);
-        case 2: return launch_r<2>(d, max_class_slices, t0, n_sweeps, st);
-        case 4: return launch_r<4>(d, max_class_slices, t0, n_sweeps, st);
+        case 1: return wide ? launch_r<1, true>(d, max_class_slices, t0, n_sweeps, st)
+                            : launch_r<1, false>(d, max_class_slices, t0, n_sweeps, st);
+        case 2: return wide ? launch_r<2, true>(d, max_class_slices, t0, n_sweeps, st)
+                            : launch_r<2, false>(d, max_class_slices, t0, n_sweeps, st);
+        case 4: return wide ? launch_r<4, true>(d, max_class_slices, t0, n_sweeps, st)
+                            : launch_r<4, false>(d, max_class_slices, t0, n_sweeps, st);
         default: return -1;
     }
 }
