@@ -372,14 +372,18 @@ public:
     }
 
     // The packed sweeps of a call, without a captured graph: a launch takes as many sweeps as run in a few
-    // milliseconds, so nothing is left of the launches' gaps.
+    // milliseconds, so nothing is left of the launches' gaps.  A single sweep is done grid-wide, whatever the
+    // form: taking the instance into shared memory and the words back costs more than the sweep saves
+    // (us a call of one sweep, shared memory against grid: N = 1000 20, 12 with one replica and 27, 17 with
+    // four; N = 14000, two replicas 29, 17; 140 graphs of 1000, four replicas 30, 25; of two sweeps 27, 27 and 35,
+    // 31; 39, 31; 37, 46).
     bool sweep_direct(int64_t t0, int64_t n, cudaStream_t st) override {
         if (kernel_ != SG_VB_PACKED) return false;
         const int64_t most = std::max<int64_t>(1, std::min<int64_t>(1024, ((int64_t)1 << 28) / (n_slots_ * R)));
         for (int64_t done = 0; done < n;) {
             const int m = (int)std::min<int64_t>(n - done, most);
             const uint32_t t = (uint32_t)(t0 + done);
-            const int k = form_ == kResident ? vb_resident_sweeps(pk_, rs_, t, m, st)
+            const int k = form_ == kResident && m > 1 ? vb_resident_sweeps(pk_, rs_, t, m, st)
                                              : vb_packed_sweeps(pk_, max_class_slices_, t, m, st);
             if (k < 0) fail(SG_ECUDA, "sweep launch failed");
             launches += k;

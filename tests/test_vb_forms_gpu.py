@@ -1,6 +1,7 @@
 """Which form a Viana-Bray handle's sweeps take: a sweep of a graph takes no longer than one of a graph of
-the same kind and twice its size, by a quarter at most, whichever of them run in shared memory; spins on
-both sides of the line between a cluster and the grid equal the oracle's."""
+the same kind and twice its size, by a quarter at most, whichever of them run in shared memory, and so
+does a call of a single sweep; spins on both sides of the line between a cluster and the grid equal the
+oracle's, also where calls of one sweep and of several alternate."""
 import numpy as np
 import pytest
 
@@ -50,6 +51,21 @@ def test_a_sweep_takes_no_longer_than_one_of_twice_the_vertices(sg, R):
         run.close()
     for n in list(t)[:-1]:
         assert t[n] <= 1.25 * t[2 * n], t
+
+
+@pytest.mark.parametrize("R", [1, 2, 4])
+def test_a_call_of_one_sweep_takes_no_longer_than_for_four_times_the_vertices(sg, R):
+    t = {}
+    for n in (1000, 3000, 12000, 48000):
+        rp, col, eid = sg_inputs.poisson_graph(n, 4.0, 7)
+        jb = sg_inputs.vb_lane_couplings(eid, int(eid.max()) + 1, 7)
+        run = sg.VBRun([dict(row_ptr=rp, col=col, jbits=jb, seed=7, temps=TEMPS[:R])], n_lanes=64, n_replicas=R)
+        run.sweep(4)
+        t[n] = us(lambda: [run.sweep(1) for _ in range(32)], 32)
+        run.synchronize()
+        run.close()
+    for n, m in zip(list(t)[:-1], list(t)[1:]):
+        assert t[n] <= 1.25 * t[m], t
 
 
 @pytest.mark.parametrize("R", [1, 2, 4])
