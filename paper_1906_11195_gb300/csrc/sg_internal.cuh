@@ -160,6 +160,9 @@ constexpr uint32_t kOrigMask = (1u << kDegShift) - 1u;
 // Slots are ordered by (colour, graph, degree descending, original label); every (colour, graph) group is
 // padded to a multiple of 32 slots, so a warp-sized slice has one colour and one graph.
 // ---------------------------------------------------------------------------------------------
+constexpr int kVbMaxColours = 64;  // greedy colouring with degree <= 63
+constexpr int kVbClaimGroups = 8;  // CTAs that share a counter of claimed slices: those of equal index mod 8
+
 struct VbPackedDev {
     const uint32_t* vinfo;       // [n_slots] orig | deg << 26, kInactive for padding slots
     const uint32_t* slice_base;  // [n_slices+1] first entry of each slice (entries of 32 lanes)
@@ -171,6 +174,7 @@ struct VbPackedDev {
     const uint4* slice_meta;     // [n_slices] {first entry, width, graph, 0}
     int* err;                    // device status word (bounded waits)
     uint32_t* gbar;              // [2] grid-barrier arrivals and exits of a sweep launch (zeroed)
+    uint32_t* claims;            // [kVbClaimGroups][2][kVbMaxColours] slices claimed in a sweep launch (zeroed)
     uint64_t* S;                 // [n_slots][R]
     uint64_t* snap;              // [n_tw][n_slots][R]
     // upper entries for the energy: per slice, each lane's neighbours in later colour classes
@@ -188,10 +192,9 @@ struct VbPackedDev {
     uint32_t max_width;          // entries of the widest slice
     const uint32_t* class_slice; // [n_colours+1] first slice of each colour class
     bool stream_first;           // the graph does not fit L2 beside the spins: its lines leave first
+    bool far_beyond_l2;          // the spins alone are a third larger than L2
     uint64_t stage_wait_ns;      // bound of one wait at the sweeps' grid barrier
 };
-
-constexpr int kVbMaxColours = 64;  // greedy colouring with degree <= 63
 
 // Viana-Bray plain layout (one graph, colour-major CSR, int8 spins per lane).
 struct VbPlainDev {

@@ -244,6 +244,7 @@ public:
             up((void*)pk_.slice_meta, h_slice_meta_.data(), h_slice_meta_.size() * sizeof(uint4));
             check_cuda(cudaMemsetAsync(pk_.err, 0, 4, st), "memset");
             check_cuda(cudaMemsetAsync(pk_.gbar, 0, 8, st), "memset");
+            check_cuda(cudaMemsetAsync(pk_.claims, 0, (size_t)kVbClaimGroups * 2 * kVbMaxColours * 4, st), "memset");
             up((void*)rs_.graph_class_slice, graph_class_slice_.data(), graph_class_slice_.size() * 4);
             up((void*)pk_.class_slice, colour_slice_.data(), colour_slice_.size() * 4);
             up((void*)pk_.jb, h_jb_.data(), h_jb_.size() * 8);
@@ -651,9 +652,11 @@ private:
             pk_.slice_meta = c.take<uint4>(h_slice_meta_.size());
             pk_.err = c.take<int>(1);
             pk_.gbar = c.take<uint32_t>(2);
+            pk_.claims = c.take<uint32_t>((size_t)kVbClaimGroups * 2 * kVbMaxColours);
             rs_.graph_class_slice = c.take<uint32_t>(graph_class_slice_.size());
             pk_.class_slice = c.take<uint32_t>(colour_slice_.size());
-            // about 96 MB of the 129 MB L2 for graph and spins together
+            // of the 129 MB L2 about 96 MB for graph and spins together
+            pk_.far_beyond_l2 = (size_t)n_slots_ * 8 * R > ((size_t)176 << 20);
             pk_.stream_first = h_col_.size() * 12 + (size_t)n_slots_ * (4 + 8 * R) > ((size_t)96 << 20);
             pk_.jb = c.take<uint64_t>(h_jb_.size());
             pk_.seeds = c.take<uint64_t>(n_inst);

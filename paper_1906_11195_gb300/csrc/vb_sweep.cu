@@ -29,12 +29,15 @@ namespace sg {
 
 namespace {
 
-// threads of a CTA (two CTAs share an SM) and entries per chunk; four replicas with chunks of 8 need
-// 255 registers (128 threads: N = 20011 16.1 us a sweep, N = 10^5 23.3; 192 threads with spills 17.4,
-// 25.9)
-template <int R, int CH>
+constexpr uint32_t kClaimGroups = kVbClaimGroups;
+
+// Threads of a CTA (two CTAs share an SM), for chunks of CH entries, without and with claimed slices.
+// Beyond L2 no register may spill: the spilled words go to HBM with the rest (N = 2^23, R = 2: 32 bytes a thread
+// 402 us a sweep, none 286).  Four replicas with chunks of 8 need 226 registers (128 threads: N = 20011 16.1 us
+// a sweep, N = 10^5 23.3; 192 threads with spills 17.4, 25.9), with chunks of 4 160.
+template <int R, int CH, bool kClaims>
 struct SweepShape {
-    static constexpr int threads = CH == 8 ? (R == 4 ? 128 : 256) : R == 1 ? 384 : R == 2 ? 320 : 256;
+    static constexpr int threads = CH == 8 ? (R == 4 ? 128 : 256) : R == 1 ? 384 : R == 4 ? 192 : kClaims ? 256 : 320;
 };
 
 constexpr int kSweepTables = 32;  // graphs whose thresholds are kept in shared memory
@@ -66,11 +69,12 @@ __device__ __forceinline__ SpinWords<R> ld_spins(const uint64_t* p, uint64_t pol
     SpinWords<R> s;
     if constexpr (R == 1) {
         asm volatile("ld.global.cg.L2::cache_hint.u64 %0, [%1], %2;" : "=l"(s.v[0]) : "l"(p), "l"(pol) : "memory");
-    } else {
-#pragma unroll
-        for (int h = 0; h < R / 2; ++h)
-            asm volatile("ld.global.cg.L2::cache_hint.v2.u64 {%0, %1}, [%2], %3;"
-                         : "=l"(s.v[2 * h]), "=l"(s.v[2 * h + 1]) : "l"(p + 2 * h), "l"(pol) : "memory");
+    } else if constexpr (R == 2) {
+        asm volatile("ld.global.cg.L2::cache_hint.v2.u64 {%0, %1}, [%2], %3;"
+                     : "=l"(s.v[0]), "=l"(s.v[1]) : "l"(p), "l"(pol) : "memory");
+    } else {  // a whole sector in one request (N = 2^22: 271 -> 210 us a sweep)
+        asm volatile("ld.global.cg.L2::cache_hint.v4.b64 {%0, %1, %2, %3}, [%4], %5;"
+                     : "=l"(s.v[0]), "=l"(s.v[1]), "=l"(s.v[2]), "=l"(s.v[3]) : "l"(p), "l"(pol) : "memory");
     }
     return s;
 }
@@ -78,10 +82,28 @@ __device__ __forceinline__ SpinWords<R> ld_spins(const uint64_t* p, uint64_t pol
 // Acceptance of one vertex: one Philox block per (vertex, sweep) serves replicas 0..3; the accepted
 // m form a prefix 1..m*, so a lane flips iff its unsatisfied count u reaches ceil((d - m*) / 2).
 // The first three thresholds come in one load (thr: shared or global memory); few draws pass all
-// three.
+// three.  Flips holds that count for each replica, at most 32, in a byte each where registers are short.
+template <int R, bool kPacked>
+struct Flips {
+    int v[R];
+    __device__ __forceinline__ void clear() {
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = 0;
+    }
+    __device__ __forceinline__ void set(int r, int k) { v[r] = k; }
+    __device__ __forceinline__ int from(int r) const { return v[r]; }
+};
 template <int R>
+struct Flips<R, true> {
+    uint32_t v;
+    __device__ __forceinline__ void clear() { v = 0u; }
+    __device__ __forceinline__ void set(int r, int k) { v = (r == 0 ? 0u : v) | (uint32_t)k << (8 * r); }
+    __device__ __forceinline__ int from(int r) const { return (int)((v >> (8 * r)) & 255u); }
+};
+
+template <int R, bool kPacked>
 __device__ __forceinline__ void accept_from(uint32_t vi, uint32_t t, uint64_t seed,
-                                            const uint32_t* thr, int (&kmin)[R]) {
+                                            const uint32_t* thr, Flips<R, kPacked>& flips) {
     const int deg = vi == kInactive ? 0 : (int)(vi >> kDegShift);
     const uint4 rnd = philox4x32_10(make_uint4(vi & kOrigMask, t, 0u, 0u), (uint32_t)seed,
                                     (uint32_t)(seed >> 32));
@@ -93,7 +115,7 @@ __device__ __forceinline__ void accept_from(uint32_t vi, uint32_t t, uint64_t se
         if (ms == 3)
             while (ms < deg && r32 < thr[r * kVbThrStride + ms + 1]) ++ms;
         ms = ms < deg ? ms : deg;
-        kmin[r] = (deg - ms + 1) >> 1;
+        flips.set(r, (deg - ms + 1) >> 1);
     }
 }
 
@@ -103,15 +125,15 @@ __device__ __forceinline__ uint32_t ld_acquire_u32(const uint32_t* p) {
     return v;
 }
 
-// the position of a warp in the sequence (sweep, class, slice)
+// the position of a warp in the sequence (sweep, class, slice); had: not its first slice of the class
 struct Cursor {
-    uint32_t sweep, cls, slice;
+    uint32_t sweep, cls, slice, had;
 };
 
 }  // namespace
 
-template <int R, int kChunk, bool kWide>
-__global__ void __launch_bounds__(SweepShape<R, kChunk>::threads, 2)
+template <int R, int kChunk, bool kWide, bool kClaims>
+__global__ void __launch_bounds__(SweepShape<R, kChunk, kClaims>::threads, 2)
     k_vb_sweeps(VbPackedDev d, uint32_t t0, uint32_t n_sweeps) {
     __shared__ uint32_t cs[kVbMaxColours + 1];  // first slice of each class
     __shared__ int s_ok;
@@ -151,7 +173,30 @@ __global__ void __launch_bounds__(SweepShape<R, kChunk>::threads, 2)
                 ++c.sweep;
             }
             c.slice = first_slice(c.cls);
+            c.had = 0u;
         }
+    };
+    // Claimed slices.  Of a class of more than two slices a warp, every warp takes its first two as ever and
+    // claims the others: number v of group g is slice 2 stride + v kClaimGroups + g.  The claim is asked for
+    // a slice before it is needed.  Every warp of a group ends a class with one claim that fails, so a class
+    // moves its counter by the same amount in every sweep.  Counters of odd and even sweeps: a warp may
+    // ask for a class's next sweep before others have ended it in this one, but not two sweeps ahead.
+    const uint32_t group = blockIdx.x % kClaimGroups;
+    const uint32_t group_warps = warps * ((gridDim.x - group + kClaimGroups - 1u) / kClaimGroups);
+    uint32_t claim = 0u;  // lane 0
+    auto claims = [&](const Cursor& c) -> bool {
+        return kClaims && gridDim.x >= kClaimGroups && c.sweep < n_sweeps && c.had > 0u && c.cls < tail &&
+               cs[c.cls + 1] - cs[c.cls] > 2u * stride + kClaimGroups;
+    };
+    auto ask = [&](const Cursor& c) {
+        if (claims(c) && lane == 0)
+            claim = atomicAdd(d.claims + (group * 2u + (c.sweep & 1u)) * kVbMaxColours + c.cls, 1u);
+    };
+    auto claimed_slice = [&](const Cursor& c) -> uint32_t {
+        const uint32_t size = cs[c.cls + 1] - cs[c.cls];
+        const uint32_t a_sweep = (size - 2u * stride - group + kClaimGroups - 1u) / kClaimGroups + group_warps;
+        const uint32_t v = __shfl_sync(0xFFFFFFFFu, claim, 0) - (c.sweep >> 1) * a_sweep;
+        return v < size ? cs[c.cls] + 2u * stride + v * kClaimGroups + group : cs[c.cls + 1];
     };
     auto load_meta = [&](const Cursor& c) -> uint4 {
         return c.sweep < n_sweeps ? __ldg(d.slice_meta + c.slice) : make_uint4(0u, 0u, 0u, 0u);
@@ -159,13 +204,24 @@ __global__ void __launch_bounds__(SweepShape<R, kChunk>::threads, 2)
 
     // the next slice: position, {first entry, width, graph}, label and degree, own words, the
     // first chunk's neighbour slots and couplings
-    Cursor nx{0u, 0u, first_slice(0)};
+    Cursor nx{0u, 0u, first_slice(0), 0u};
     settle(nx);
     uint4 nm = load_meta(nx);
     Cursor nn = nx;  // the one after, of which only the meta data is read ahead
     auto step = [&](Cursor& c) {
-        c.slice += c.cls < tail ? stride : warps;
-        settle(c);
+        if constexpr (kClaims) {
+            if (claims(c)) {
+                c.slice = claimed_slice(c);
+            } else {
+                c.slice += c.cls < tail ? stride : warps;
+                c.had = 1u;
+            }
+            settle(c);
+            ask(c);
+        } else {
+            c.slice += c.cls < tail ? stride : warps;
+            settle(c);
+        }
     };
     step(nn);
     uint4 nnm = load_meta(nn);
@@ -176,7 +232,8 @@ __global__ void __launch_bounds__(SweepShape<R, kChunk>::threads, 2)
     SpinWords<R> nsi;
     uint32_t col[kChunk];
     uint64_t J[kChunk];
-    int nkmin[R];
+    Flips<R, kClaims> nflips;
+    nflips.clear();
 #pragma unroll
     for (int e = 0; e < kChunk; ++e) {
         col[e] = 0u;
@@ -185,7 +242,6 @@ __global__ void __launch_bounds__(SweepShape<R, kChunk>::threads, 2)
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         nsi.v[r] = 0ull;
-        nkmin[r] = 0;
     }
     auto load_chunk = [&](uint32_t idx, uint32_t n) {
 #pragma unroll
@@ -206,7 +262,7 @@ __global__ void __launch_bounds__(SweepShape<R, kChunk>::threads, 2)
     };
     auto next_acceptance = [&] {
         if (nx.sweep < n_sweeps)
-            accept_from<R>(nvi, t0 + nx.sweep, seeds[nm.z], thr + nm.z * (R * kVbThrStride), nkmin);
+            accept_from(nvi, t0 + nx.sweep, seeds[nm.z], thr + nm.z * (R * kVbThrStride), nflips);
     };
     load_slice();
 
@@ -214,6 +270,13 @@ __global__ void __launch_bounds__(SweepShape<R, kChunk>::threads, 2)
     uint32_t sweep = 0, cls = 0, phase = 0;  // phases: spans between grid-wide barriers
     bool ok = true;
     for (uint32_t q = 0; q < nq; ++q) {
+        // beside claims there are registers to work out the next acceptance while gathers are on their way, but
+        // for wide slices it waits (512 graphs of 84 M vertices 3.12 ms, for all slices early 3.38)
+        auto next_early = [&] {
+            if constexpr (kClaims) {
+                if (nx.sweep == sweep && nx.cls == cls) next_acceptance();
+            }
+        };
         if (nx.sweep == sweep && nx.cls == cls) next_acceptance();
         if (phase > 0 && cls <= tail && gridDim.x > 1) {
             // admitted once every CTA has written the classes before (bounded).  Acquiring polls: the
@@ -246,16 +309,15 @@ __global__ void __launch_bounds__(SweepShape<R, kChunk>::threads, 2)
         while (nx.sweep == sweep && nx.cls == cls) {
             const uint32_t slice = nx.slice, vi = nvi;
             SpinWords<R> si = nsi;
-            int kmin[R];
-#pragma unroll
-            for (int r = 0; r < R; ++r) kmin[r] = nkmin[r];
+            const Flips<R, kClaims> flips = nflips;
             uint32_t left = nm.y, idx = nm.x + lane;
             auto advance = [&] {
                 nx = nn;
                 nm = nnm;
                 nvi = nnvi;
-                step(nn);
+                if constexpr (!kClaims) step(nn);
                 load_slice();
+                if constexpr (kClaims) step(nn);  // may wait for its claim
                 nnm = load_meta(nn);
                 nnvi = load_vi(nn);
             };
@@ -282,6 +344,7 @@ __global__ void __launch_bounds__(SweepShape<R, kChunk>::threads, 2)
                         load_chunk(idx, left);
                     } else {
                         advance();
+                        if constexpr (kClaims && P == kSweepPlanes) next_early();
                     }
 #pragma unroll
                     for (int r = 0; r < R; ++r) {
@@ -294,15 +357,20 @@ __global__ void __launch_bounds__(SweepShape<R, kChunk>::threads, 2)
                     if (last) break;
                 }
 #pragma unroll
-                for (int r = 0; r < R; ++r) si.v[r] ^= at_least<P>(p[r], kmin[r]);
+                for (int r = 0; r < R; ++r) si.v[r] ^= at_least<P>(p[r], flips.from(r));
             };
             if (!kWide || left < (1u << kSweepPlanes)) count(std::integral_constant<int, kSweepPlanes>{});
-            else if constexpr (kWide) count(std::integral_constant<int, kSweepWidePlanes>{});
+            else if constexpr (kWide) {
+                count(std::integral_constant<int, kSweepWidePlanes>{});
+                if constexpr (kClaims) next_early();
+            }
             // a warp's only slice comes next again: its words were read ahead of this update
             if (nx.slice == slice) nsi = si;
             if (vi != kInactive)
                 store_words_keep<R>(d.S + ((int64_t)slice * 32 + lane) * R, si, pol_keep);
-            if (nx.sweep == sweep && nx.cls == cls) next_acceptance();
+            if constexpr (!kClaims) {
+                if (nx.sweep == sweep && nx.cls == cls) next_acceptance();
+            }
         }
         __syncthreads();  // this CTA's words of the class are written
         if (tail <= cls && cls + 1 < nc) {  // the tail goes on
@@ -324,18 +392,21 @@ __global__ void __launch_bounds__(SweepShape<R, kChunk>::threads, 2)
         if (atomicAdd(d.gbar + 1, 1u) == gridDim.x - 1) {
             atomicExch(d.gbar, 0u);
             atomicExch(d.gbar + 1, 0u);
+            if constexpr (kClaims)
+                for (uint32_t g = 0; g < 2u * kClaimGroups; ++g)
+                    for (uint32_t c = 0; c < nc; ++c) d.claims[g * kVbMaxColours + c] = 0u;
         }
     }
 }
 
 template <int R, int CH>
-static int sweep_warps(int sms) { return SweepShape<R, CH>::threads / 32 * 2 * sms; }
+static int sweep_warps(int sms) { return SweepShape<R, CH, false>::threads / 32 * 2 * sms; }
 
-template <int R, int CH, bool kWide>
+template <int R, int CH, bool kWide, bool kClaims>
 static int launch_sweeps(const VbPackedDev& d, int max_class_slices, int sms, uint32_t t0,
                          int n_sweeps, cudaStream_t st) {
-    constexpr int threads = SweepShape<R, CH>::threads, warps = threads / 32;
-    auto kern = k_vb_sweeps<R, CH, kWide>;
+    constexpr int threads = SweepShape<R, CH, kClaims>::threads, warps = threads / 32;
+    auto kern = k_vb_sweeps<R, CH, kWide, kClaims>;
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, 0) != cudaSuccess ||
         per_sm < 1)
@@ -364,6 +435,13 @@ static int launch_sweeps(const VbPackedDev& d, int max_class_slices, int sms, ui
 // N = 65536: 15.6 us a sweep, 16.6 with chunks of 4; R = 4, N = 60000: 23.3, 27.1).  Beyond that the
 // registers are better spent on more warps (R = 2, bipartite N = 2^18: 10.3 us with chunks of 4,
 // 11.9 with 8; Poissonian N = 2^22: 128, 145; R = 4, N = 10^6: 80, 90).
+// Slices are claimed far beyond L2.  There SMs differ by a fifth in what HBM gives them, and with the same slices
+// for every warp a CTA stood still for 9 % of the time at the end of a class, on average (R = 2, N = 2^24
+// 958 us a sweep, claimed 903; 12 2^20 581, 562; 512 graphs of 84 M vertices 3.41 ms, 3.12).  Nearer to L2 two
+// replicas need the fifth warp of each scheduler as much (2^23 283, claimed 285; 2^22 122, 127); one replica
+// has six and does not gain (2^24 466, claimed 647 with five); four replicas run three without spills either
+// way, and claim everywhere (N = 2^20 53, claimed 54; 2^22 209, 199; 2^23 558, 526).  One counter for all CTAs is too
+// few (2^24 1069), 32 are too many, as each serves few CTAs (942; 4 to 16 903 to 908).
 template <int R, bool kWide>
 static int launch_r(const VbPackedDev& d, int max_class_slices, uint32_t t0, int n_sweeps, cudaStream_t st) {
     int dev = 0, sms = 0;
@@ -371,8 +449,11 @@ static int launch_r(const VbPackedDev& d, int max_class_slices, uint32_t t0, int
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
         return -1;
     if (max_class_slices <= sweep_warps<R, 8>(sms))
-        return launch_sweeps<R, 8, kWide>(d, max_class_slices, sms, t0, n_sweeps, st);
-    return launch_sweeps<R, 4, kWide>(d, max_class_slices, sms, t0, n_sweeps, st);
+        return launch_sweeps<R, 8, kWide, false>(d, max_class_slices, sms, t0, n_sweeps, st);
+    if constexpr (R >= 2) {
+        if (R == 4 || d.far_beyond_l2) return launch_sweeps<R, 4, kWide, true>(d, max_class_slices, sms, t0, n_sweeps, st);
+    }
+    if constexpr (R <= 2) return launch_sweeps<R, 4, kWide, false>(d, max_class_slices, sms, t0, n_sweeps, st);
 }
 
 int vb_packed_sweeps(const VbPackedDev& d, int max_class_slices, uint32_t t0, int n_sweeps,
