@@ -190,6 +190,7 @@ struct VbPackedDev {
     int32_t n_colours;
     int32_t n_graphs;
     uint32_t max_width;          // entries of the widest slice
+    uint32_t n_rows;             // rows of 32 entries
     const uint32_t* class_slice; // [n_colours+1] first slice of each colour class
     bool stream_first;           // the graph does not fit L2 beside the spins: its lines leave first
     bool far_beyond_l2;          // the spins alone are a third larger than L2

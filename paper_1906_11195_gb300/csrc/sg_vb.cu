@@ -675,6 +675,7 @@ private:
             pk_.R = R;
             pk_.n_graphs = n_inst;
             pk_.max_width = max_width_;
+            pk_.n_rows = (uint32_t)(h_col_.size() / 32);
             pk_.n_colours = (int32_t)colour_slice_.size() - 1;
             // SG_TEST_STAGE_WAIT_NS shortens the colour kernel's pipeline waits: a test of the
             // timeout path (the kernel gives up, flags SG_ETIMEOUT and exits cleanly)

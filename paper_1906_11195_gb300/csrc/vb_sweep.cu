@@ -434,7 +434,9 @@ static int launch_sweeps(const VbPackedDev& d, int max_class_slices, int sms, ui
 // as its widest slice, and fewer rounds of gathers count for more than warps in flight (R = 2,
 // N = 65536: 15.6 us a sweep, 16.6 with chunks of 4; R = 4, N = 60000: 23.3, 27.1).  Beyond that the
 // registers are better spent on more warps (R = 2, bipartite N = 2^18: 10.3 us with chunks of 4,
-// 11.9 with 8; Poissonian N = 2^22: 128, 145; R = 4, N = 10^6: 80, 90).
+// 11.9 with 8; Poissonian N = 2^22: 128, 145; R = 4, N = 10^6: 80, 90), except for one replica of a graph whose
+// slices have eight entries or more on average (N = 2^20, mean degree 8 65, with chunks of 4 67; 12 86, 94;
+// 16 111, 125; degree 6 45, 46).
 // Slices are claimed far beyond L2.  There SMs differ by a fifth in what HBM gives them, and with the same slices
 // for every warp a CTA stood still for 9 % of the time at the end of a class, on average (R = 2, N = 2^24
 // 958 us a sweep, claimed 903; 12 2^20 581, 562; 512 graphs of 84 M vertices 3.41 ms, 3.12).  Nearer to L2 two
@@ -448,7 +450,7 @@ static int launch_r(const VbPackedDev& d, int max_class_slices, uint32_t t0, int
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
         return -1;
-    if (max_class_slices <= sweep_warps<R, 8>(sms))
+    if (max_class_slices <= sweep_warps<R, 8>(sms) || (R == 1 && d.n_rows >= 8u * (uint32_t)d.n_slices))
         return launch_sweeps<R, 8, kWide, false>(d, max_class_slices, sms, t0, n_sweeps, st);
     if constexpr (R >= 2) {
         if (R == 4 || d.far_beyond_l2) return launch_sweeps<R, 4, kWide, true>(d, max_class_slices, sms, t0, n_sweeps, st);

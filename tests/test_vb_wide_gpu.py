@@ -42,7 +42,7 @@ def instance(graph, z, R):
 
 @pytest.mark.parametrize("R", [1, 2, 4])
 @pytest.mark.parametrize("n,z", [(n, z) for n in (200, 3000, 30000) for z in (15, 16, 17, 20, 24, 25, 31, 32, 63)] +
-                         [(250_000, 17), (250_000, 25)])
+                         [(250_000, 17), (250_000, 25), (400_000, 7), (400_000, 9)])
 def test_spins(sg, n, z, R):
     g = instance(circulant(n, z), z, R)
     run = sg.VBRun([g], n_lanes=64, n_replicas=R)
