@@ -323,10 +323,11 @@ public:
     // With copies of all words a CTA sends each slice that it updates to the others; without, it gathers
     // its slices' entries, a row of 32 at a time, from them.  Examples (us a sweep, one replica where not
     // said, cluster against grid): bipartite N = 8192 3.6, 4.0; 16384 5.7, 4.1; 32768 13.5, 4.2; two replicas
-    // 4096 3.0, 4.5; 16384 7.8, 4.6; four replicas 4096 4.8, 4.9; 8192 8.2, 4.9; Poissonian of degree 4,
-    // N = 16384 8.1, 10.9; 24000 14.5, 11.6; nine bipartite graphs of 9000, two replicas, 6.0, 6.8.
+    // 4096 3.0, 4.5; 16384 7.8, 4.6; four replicas 4096 4.8, 4.9; 8192 8.2, 4.9; eight Poissonian graphs of degree 4,
+    // N = 5000, 13.0, 14.8; one of them, one replica, N = 16384 8.1, 10.9; 24000 14.5, 11.6; nine bipartite graphs of
+    // 9000, two replicas, 6.0, 6.8.
     double cluster_us(const VbResident& rs, int64_t graph_entries, int more) const {
-        static const double kCopies[3][3] = {{0.8, 0.03, 0.0065}, {0.75, 0.04, 0.0125}, {1.5, 0.06, 0.04}};
+        static const double kCopies[3][3] = {{0.8, 0.03, 0.0065}, {0.75, 0.04, 0.0125}, {1.5, 0.132, 0.017}};
         static const double kGather[3][3] = {{0.95, 0.045, 0.15}, {0.85, 0.047, 0.25}, {0.9, 0.096, 0.6}};
         const int q = R == 4 ? 2 : R - 1;
         const double slices = (double)rs.max_slices / pk_.n_colours;
