@@ -128,16 +128,6 @@ __device__ __forceinline__ void bulk_copy_g2s(void* dst, const void* src, uint32
         : "memory");
 }
 
-// Same, with an L2 cache-policy operand (createpolicy) attached to the copy.
-__device__ __forceinline__ void bulk_copy_g2s_hint(void* dst, const void* src, uint32_t bytes,
-                                                   uint64_t* bar, uint64_t policy) {
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
-        " [%0], [%1], %2, [%3], %4;" ::"r"(smem_addr(dst)),
-        "l"(reinterpret_cast<uint64_t>(src)), "r"(bytes), "r"(smem_addr(bar)), "l"(policy)
-        : "memory");
-}
-
 // L2 eviction-priority policies: streamed data goes first, the spin array stays
 __device__ __forceinline__ uint64_t l2_evict_first() {
     uint64_t p;

@@ -678,8 +678,8 @@ private:
             pk_.max_width = max_width_;
             pk_.n_rows = (uint32_t)(h_col_.size() / 32);
             pk_.n_colours = (int32_t)colour_slice_.size() - 1;
-            // SG_TEST_STAGE_WAIT_NS shortens the colour kernel's pipeline waits: a test of the
-            // timeout path (the kernel gives up, flags SG_ETIMEOUT and exits cleanly)
+            // SG_TEST_STAGE_WAIT_NS shortens the waits at the grid-wide barrier: a test of the timeout
+            // path (the kernel gives up, flags SG_ETIMEOUT and exits cleanly)
             pk_.stage_wait_ns = 2000000000ull;
             if (const char* w = getenv("SG_TEST_STAGE_WAIT_NS")) pk_.stage_wait_ns = strtoull(w, nullptr, 10);
             if (pk_.n_colours > kVbMaxColours) fail(SG_EINVAL, "more colour classes than supported");
