@@ -224,11 +224,15 @@ int vb_packed_measure(const VbPackedDev& d, const VbMeasure& m, cudaStream_t st)
     if (rows == 0) return 0;
     MeasureGrid mg;
     mg.up_rows = d.up_rows;
-    // Whole waves of the CTAs that the 152 SMs hold at once.  In one or two waves the slowest run is the
+    // Whole waves of the CTAs that the SMs hold at once.  In one or two waves the slowest run is the
     // time: a row of edges takes longer than a row of spins (its gathers wait for its slots), so its
     // runs are half as long (five snapshots, N = 2^20: 72 -> 60 us; a third as long 61, a quarter 65).
     // More waves even out by themselves (N = 2^22: 180 us, with shorter edge runs 185).
-    const int64_t slots = 152 * (d.R == 4 ? kMeasureCtas<4> : kMeasureCtas<2>);
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1)
+        return -1;
+    const int64_t slots = (int64_t)sms * (d.R == 4 ? kMeasureCtas<4> : kMeasureCtas<2>);
     auto waves_of = [&](int64_t c) { return (c + slots * kMeasureWarps * kMeasureRun - 1) / (slots * kMeasureWarps * kMeasureRun); };
     const int64_t edge_cost = waves_of(rows) <= 2 ? 2 : 1;
     const int64_t cost = (int64_t)d.n_slices * passes + (m.e ? (int64_t)d.up_rows * edge_cost : 0);
