@@ -15,8 +15,8 @@
 // where the copies fit it is cheaper to send every updated slice to the other CTAs (512 bytes for two
 // replicas, whole lines, about 43 cycles each) and gather at home.
 //
-// us a sweep, two replicas, before (grid-wide) -> now: N = 1000 18 -> 4.5 (one CTA), 2500 12.4 -> 5.0,
-// bipartite 4096 9.8 -> 2.9, 6000 14 -> 6.4, 9000 15 -> 8.1.
+// us a sweep, two replicas, before (grid-wide) -> now: N = 1000 18 -> 4.4 (one CTA), 2500 12.4 -> 4.9,
+// bipartite 4096 9.8 -> 2.9, 6000 14 -> 6.4, 9000 15 -> 8.0.
 //
 // The slices (32 vertices) of a class are dealt in turn to the CTAs of the cluster, and in a CTA to
 // its warps.

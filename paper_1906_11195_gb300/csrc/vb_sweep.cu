@@ -3,21 +3,23 @@
 // colour class (an independent set) at a time, the generalisation of the bipartite half-updates of
 // SI section 3, with a grid-wide barrier between classes.
 //
-// A warp owns the same slices (32 vertices of one class, degree-sorted) in every sweep.  Its work is
-// a chain of chunks of four (or eight) sliced-ELL entries: while the neighbours' words of one chunk are on
-// their way from L2, the neighbour slots and coupling words of the next chunk (of the next slice,
-// the next class or the next sweep: nothing a sweep writes, except a vertex's own words, which only
-// this thread writes) are already being read into registers, and the next slice's random numbers
-// and acceptance thresholds are worked out before the barrier that admits its gathers.
+// A warp owns the same slices (32 vertices of one class, degree-sorted) in every sweep, or, far beyond L2
+// and with four replicas, its first two of a class, and claims the others.  Its work is a chain of chunks of
+// four (or eight) sliced-ELL entries: while the neighbours' words of one chunk are on their way from L2, the
+// neighbour slots and coupling words of the next chunk (of the next slice, the next class or the next sweep)
+// are already being read into registers: nothing a sweep writes, except a vertex's own words, which only
+// this thread writes or, in a claimed slice, another one before a barrier that was passed.  The next slice's
+// random numbers and acceptance thresholds are worked out before the barrier that admits its gathers.
 //
-// What bounds it.  Small and middling graphs: a class takes about 2.3 us of latencies (the stores'
+// What bounds it.  Small and middling graphs: a class takes about 2.1 us of latencies (the stores'
 // release, the barrier's way through L2 and back, a gather) before any work.  Large ones: a sweep
-// of N = 2^22 (degree 4, two replicas) reads 84 bytes per vertex from HBM (31 % of its peak), gathers
-// 16.8 million word pairs, each a 32-byte sector of L2 (45 %) and a tag of L1 (50 %), and issues 515
-// instructions per slice (41 %).  us a sweep, before (groups staged by bulk copies into shared-memory
-// rings, a launch per sweep) -> now: N = 2^22 131 -> 128, 2^20 50 -> 39, bipartite 2^18 14.2 -> 9.6,
-// N = 300007 with one replica (a launch per class) 30.8 -> 16, N = 20011 with four 24.9 -> 16.1.
-// Without the rings there is no pipeline to fill and drain in each class, and no launch gap.
+// of N = 2^22 (degree 4, two replicas) reads 84 bytes per vertex from HBM (33 % of its peak), gathers
+// 16.8 million word pairs, each a 32-byte sector of L2 (47 %) and a tag of L1 (51 %), and issues 500
+// instructions per slice (42 %).  Far beyond L2 HBM: N = 2^24 moves 5.9 GB a sweep, 64 bytes for nearly every
+// gather, at 6.5 TB/s, 0.96 of the rate of a plain copy.  us a sweep, before (groups staged by bulk copies
+// into shared-memory rings, a launch per sweep) -> now: N = 2^24 950 -> 903, 2^22 129 -> 122, 2^20 49 -> 37,
+// bipartite 2^18 14.2 -> 9.5, N = 300007 with one replica (a launch per class) 30.8 -> 15, N = 20011 with
+// four 24.9 -> 14.  Without the rings there is no pipeline to fill and drain in each class, and no launch gap.
 #include <algorithm>
 #include <type_traits>
 
@@ -34,13 +36,15 @@ constexpr uint32_t kClaimGroups = kVbClaimGroups;
 // Threads of a CTA (two CTAs share an SM), for chunks of CH entries, without and with claimed slices.
 // Beyond L2 no register may spill: the spilled words go to HBM with the rest (N = 2^23, R = 2: 32 bytes a thread
 // 402 us a sweep, none 286).  Four replicas with chunks of 8 need 226 registers (128 threads: N = 20011 16.1 us
-// a sweep, N = 10^5 23.3; 192 threads with spills 17.4, 25.9), with chunks of 4 160.
+// a sweep, N = 10^5 23.3; 192 threads with spills 17.4, 25.9; since, 14.0 and 18.3), with chunks of 4 157.
 template <int R, int CH, bool kClaims>
 struct SweepShape {
     static constexpr int threads = CH == 8 ? (R == 4 ? 128 : 256) : R == 1 ? 384 : R == 4 ? 192 : kClaims ? 256 : 320;
 };
 
-constexpr int kSweepTables = 32;  // graphs whose thresholds are kept in shared memory
+// Graphs whose thresholds are kept in shared memory, 32 KB for four replicas; a batch of more reads them through
+// L1 (batches of 17 to 32 graphs gained 1.5 % from 16; more were not tried).
+constexpr int kSweepTables = 32;
 // Counter planes: slices up to width 15, and wider ones (degrees up to 63).  Both take their entries in
 // chunks: one entry at a time, each waiting for its slot and then its words, a class lasts as long as its
 // widest slice (us a sweep, one at a time -> chunks: N = 20000, degree 12, R = 2 55.8 -> 29.2, R = 4
