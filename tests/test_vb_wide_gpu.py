@@ -70,7 +70,7 @@ def us_per_sweep(sg, n, z, R, sweeps=32):
         times.append(a.elapsed_time(b) / sweeps * 1e3)
     run.synchronize()
     run.close()
-    return sorted(times)[3]
+    return min(times)  # what else the machine does only adds to them
 
 
 @pytest.mark.parametrize("R", [1, 2, 4])
